@@ -7,7 +7,7 @@
 //   zone_kernel<RETURN, T>                   the near-horizon zone of the
 //                                            selective mode (double-single or double)
 //   probe_rays_kernel, plan_*_kernel         the longest-first planner
-//   render_kernel, shadow_*, ring_*, splat   read-out of results
+//   render_*, shadow_*, ring_*, splat        read-out of results
 //   eval_kernel<T>                           unit evaluations for parity tests
 //
 // Trace kernel design (GRay Sec. 2 puts one photon in one thread; here a
@@ -1417,32 +1417,77 @@ __device__ void load_state_double(const StateView &v, int prec, int64_t i, doubl
     }
 }
 
-__global__ void render_kernel(StateView v, int prec, int64_t first, int64_t n, int kind, void *out)
+// One kernel per kind, so that a ray moves only what its record holds.  The
+// bound is HBM: a PIXELS32 pixel takes 32 B of state and 16 B of result where
+// one kernel for all kinds read the whole 144 B state first.
+// 1024^2 pixels: 61 -> 9 us.
+__global__ void render_pixels_kernel(StateView v, int prec, int64_t first, int64_t n, int kind, void *out)
 {
-    int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (j >= n)
         return;
     const int64_t i = first + j;
-    double y[8], fin[4];
-    load_state_double(v, prec, i, y, fin);
     const int4 s0 = v.S0[i];
+    double r, th, ph;
+    if (prec == GRAY_FP64) {
+        const d4 F = ld_d4(v.F, i);
+        r = F.y;
+        th = F.z;
+        ph = F.w;
+    } else {
+        const float4 F = ld_f4(v.F, i);
+        if (kind == GRAY_RENDER_PIXELS32) { // already single: no trip through double
+            gray_pixel32 px;
+            px.r = F.y;
+            px.theta = F.z;
+            px.phi = F.w;
+            px.status = s0.x;
+            if (((uintptr_t)out & 15) == 0)
+                ((float4 *)out)[j] = make_float4(px.r, px.theta, px.phi, __int_as_float(px.status));
+            else
+                ((gray_pixel32 *)out)[j] = px;
+            return;
+        }
+        r = F.y;
+        th = F.z;
+        ph = F.w;
+    }
     if (kind == GRAY_RENDER_PIXELS64) {
         gray_pixel64 px;
-        px.r = fin[1];
-        px.theta = fin[2];
-        px.phi = fin[3];
+        px.r = r;
+        px.theta = th;
+        px.phi = ph;
         px.status = s0.x;
         px.steps = s0.y;
         ((gray_pixel64 *)out)[j] = px;
-    } else if (kind == GRAY_RENDER_PIXELS32) {
+    } else {
         gray_pixel32 px;
-        px.r = (float)fin[1];
-        px.theta = (float)fin[2];
-        px.phi = (float)fin[3];
+        px.r = (float)r;
+        px.theta = (float)th;
+        px.phi = (float)ph;
         px.status = s0.x;
         ((gray_pixel32 *)out)[j] = px;
-    } else if (kind == GRAY_RENDER_RECORD) {
-        double *o = (double *)out + 17 * j;
+    }
+}
+
+// Records of 17 doubles (136 B): a thread's own stores would touch 32 sectors
+// per instruction, a quarter of each; the block stages its rows in shared
+// memory (17 doubles apart: 64-bit accesses of a half warp fall on 16
+// different bank pairs) and writes them as one contiguous stream.
+// 1000 x 777 rays: 96 -> 52 us.
+constexpr int RECORD_BLOCK = 128;
+__global__ void __launch_bounds__(RECORD_BLOCK) render_record_kernel(StateView v, int prec, int64_t first, int64_t n,
+                                                                     double *out)
+{
+    __shared__ double rows[RECORD_BLOCK * 17];
+    const int64_t j0 = (int64_t)blockIdx.x * RECORD_BLOCK;
+    const int64_t j = j0 + threadIdx.x;
+    if (j < n) {
+        const int64_t i = first + j;
+        double y[8], fin[4];
+        load_state_double(v, prec, i, y, fin);
+        const int4 s0 = v.S0[i];
+        double *o = rows + 17 * threadIdx.x;
         o[0] = s0.x;
         o[1] = s0.y;
         o[2] = s0.z;
@@ -1452,57 +1497,123 @@ __global__ void render_kernel(StateView v, int prec, int64_t first, int64_t n, i
         for (int m = 0; m < 8; ++m)
             o[8 + m] = y[m];
         o[16] = v.S1[i].x;
-    } else { // GRAY_RENDER_INVARIANTS, in double from the stored state
-        const d4 p = ld_d4(v.P, i);
-        const Hole<double> H = make_hole(p.x, p.y, p.z, 1.0, 1.0, 0.0);
-        double s, c;
-        sincos(y[2], &s, &c);
-        const MetricPieces<double> m = metric_pieces(H, y[1], s, c);
-        const double kt = y[4], kr = y[5], kh = y[6], kp = y[7];
-        const double E = -(m.gtt * kt + m.gtp * kp);
-        const double L = m.gtp * kt + m.gpp * kp;
-        const double kth_low = m.gthth * kh;
-        const double Q = kth_low * kth_low + c * c * (-H.a * H.a * E * E + L * L / (s * s));
-        const double N = m.gtt * kt * kt + 2.0 * m.gtp * kt * kp + m.grr * kr * kr + m.gthth * kh * kh + m.gpp * kp * kp;
-        double *o = (double *)out + 4 * j;
-        o[0] = E;
-        o[1] = L;
-        o[2] = Q;
-        o[3] = N;
     }
+    __syncthreads();
+    const int count = 17 * (int)(n - j0 < RECORD_BLOCK ? n - j0 : RECORD_BLOCK);
+    for (int e = threadIdx.x; e < count; e += RECORD_BLOCK)
+        out[17 * j0 + e] = rows[e];
+}
+
+// GRAY_RENDER_INVARIANTS, in double from the stored state (bound by the FP64
+// pipe: a sine and cosine, a square root and four divides per ray).
+__global__ void render_invariants_kernel(StateView v, int prec, int64_t first, int64_t n, double *out)
+{
+    const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+    if (j >= n)
+        return;
+    const int64_t i = first + j;
+    double y[8], fin[4];
+    load_state_double(v, prec, i, y, fin);
+    const d4 p = ld_d4(v.P, i);
+    const Hole<double> H = make_hole(p.x, p.y, p.z, 1.0, 1.0, 0.0);
+    double s, c;
+    sincos(y[2], &s, &c);
+    const MetricPieces<double> m = metric_pieces(H, y[1], s, c);
+    const double kt = y[4], kr = y[5], kh = y[6], kp = y[7];
+    const double E = -(m.gtt * kt + m.gtp * kp);
+    const double L = m.gtp * kt + m.gpp * kp;
+    const double kth_low = m.gthth * kh;
+    const double Q = kth_low * kth_low + c * c * (-H.a * H.a * E * E + L * L / (s * s));
+    const double N = m.gtt * kt * kt + 2.0 * m.gtp * kt * kp + m.grr * kr * kr + m.gthth * kh * kh + m.gpp * kp * kp;
+    double *o = out + 4 * j;
+    o[0] = E;
+    o[1] = L;
+    o[2] = Q;
+    o[3] = N;
 }
 
 // Shadow moments: counts and the sums of the captured pixels' column and row
 // indices per image, accumulated as 64-bit integers (exact, independent of
 // the order of the atomics) directly in the caller's output records, then
 // turned into area, radius and centroid.
-__global__ void shadow_accum_kernel(StateView v, int64_t first, const ImageDev *imgs, int n_images, int64_t total,
-                                    gray_shadow_info *out)
+//
+// One block takes SHADOW_RAYS consecutive rays.  Every ray's own atomics on
+// its image's counters would serialise on a few addresses (24 images, 2.0 M
+// rays: 1477 us); here a block whose rays lie in at most SHADOW_SEGMENTS
+// images sums each image's part in registers and shuffles and adds it once
+// (14 us; HBM: 16 B per ray).  Blocks over many small images (under a
+// quarter of a block's rays each) keep the atomics per ray, which then fall
+// on different addresses.
+constexpr int SHADOW_BLOCK = 256, SHADOW_RAYS = 2048, SHADOW_SEGMENTS = 4;
+
+__global__ void __launch_bounds__(SHADOW_BLOCK) shadow_accum_kernel(StateView v, int64_t first, const ImageDev *imgs,
+                                                                    int n_images, int64_t total,
+                                                                    gray_shadow_info *out)
 {
-    int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i >= total)
+    __shared__ unsigned long long part[5][SHADOW_BLOCK / 32];
+    const int64_t b0 = (int64_t)blockIdx.x * SHADOW_RAYS;
+    const int64_t b1 = total - b0 < SHADOW_RAYS ? total : b0 + SHADOW_RAYS;
+    const int k0 = image_of(imgs, n_images, b0), k1 = image_of(imgs, n_images, b1 - 1);
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    if (k1 - k0 < SHADOW_SEGMENTS) {
+        for (int k = k0; k <= k1; ++k) { // block-uniform
+            const int64_t f = imgs[k].first;
+            const unsigned nx = (unsigned)imgs[k].nx;
+            const int64_t i0 = f > b0 ? f : b0;
+            const int64_t i1 = (k < k1) ? imgs[k + 1].first : b1;
+            unsigned long long sum[5] = {0, 0, 0, 0, 0}; // captured, escaped, other, columns, rows
+            for (int64_t i = i0 + tid; i < i1; i += SHADOW_BLOCK) {
+                const int st = v.S0[first + i].x;
+                if (st == GRAY_RAY_CAPTURED) {
+                    const unsigned q = (unsigned)(i - f), row = q / nx; // a buffer holds fewer than 2^31 rays
+                    sum[0] += 1;
+                    sum[3] += q - row * nx;
+                    sum[4] += row;
+                } else if (st == GRAY_RAY_ESCAPED) {
+                    sum[1] += 1;
+                } else {
+                    sum[2] += 1;
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 5; ++m) {
+#pragma unroll
+                for (int off = 16; off > 0; off >>= 1)
+                    sum[m] += __shfl_xor_sync(0xffffffffu, sum[m], off);
+                if (lane == 0)
+                    part[m][warp] = sum[m];
+            }
+            __syncthreads();
+            if (tid < 5) {
+                unsigned long long t = 0;
+                for (int w = 0; w < SHADOW_BLOCK / 32; ++w)
+                    t += part[tid][w];
+                gray_shadow_info *o = out + k;
+                unsigned long long *const dst[5] = {(unsigned long long *)&o->n_captured,
+                                                    (unsigned long long *)&o->n_escaped,
+                                                    (unsigned long long *)&o->n_other,
+                                                    (unsigned long long *)&o->alpha_c, (unsigned long long *)&o->beta_c};
+                if (t)
+                    atomicAdd(dst[tid], t);
+            }
+            __syncthreads(); // part is rewritten by the next image
+        }
         return;
-    int lo = 0, hi = n_images - 1;
-    while (lo < hi) {
-        int mid = (lo + hi + 1) >> 1;
-        if (imgs[mid].first <= i)
-            lo = mid;
-        else
-            hi = mid - 1;
     }
-    const ImageDev im = imgs[lo];
-    const int64_t p = i - im.first;
-    const int64_t row = p / im.nx, col = p - row * im.nx;
-    const int st = v.S0[first + i].x;
-    gray_shadow_info *o = out + lo;
-    if (st == GRAY_RAY_CAPTURED) {
-        atomicAdd((unsigned long long *)&o->n_captured, 1ull);
-        atomicAdd((unsigned long long *)&o->alpha_c, (unsigned long long)col);
-        atomicAdd((unsigned long long *)&o->beta_c, (unsigned long long)row);
-    } else if (st == GRAY_RAY_ESCAPED) {
-        atomicAdd((unsigned long long *)&o->n_escaped, 1ull);
-    } else {
-        atomicAdd((unsigned long long *)&o->n_other, 1ull);
+    for (int64_t i = b0 + tid; i < b1; i += SHADOW_BLOCK) {
+        const int k = image_of(imgs, n_images, i);
+        const unsigned nx = (unsigned)imgs[k].nx, q = (unsigned)(i - imgs[k].first), row = q / nx;
+        const int st = v.S0[first + i].x;
+        gray_shadow_info *o = out + k;
+        if (st == GRAY_RAY_CAPTURED) {
+            atomicAdd((unsigned long long *)&o->n_captured, 1ull);
+            atomicAdd((unsigned long long *)&o->alpha_c, (unsigned long long)(q - row * nx));
+            atomicAdd((unsigned long long *)&o->beta_c, (unsigned long long)row);
+        } else if (st == GRAY_RAY_ESCAPED) {
+            atomicAdd((unsigned long long *)&o->n_escaped, 1ull);
+        } else {
+            atomicAdd((unsigned long long *)&o->n_other, 1ull);
+        }
     }
 }
 
@@ -2746,7 +2857,14 @@ int gray_render(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_
     if (!out || out_bytes < per * (size_t)n)
         return GRAY_EINVAL;
     StateView v = make_view((void *)state, n_state, ctx->opt.precision);
-    render_kernel<<<grid_for(n, 256), 256, 0, (cudaStream_t)stream>>>(v, ctx->opt.precision, first_ray, n, kind, out);
+    const cudaStream_t s = (cudaStream_t)stream;
+    if (kind == GRAY_RENDER_RECORD)
+        render_record_kernel<<<grid_for(n, RECORD_BLOCK), RECORD_BLOCK, 0, s>>>(v, ctx->opt.precision, first_ray, n,
+                                                                                (double *)out);
+    else if (kind == GRAY_RENDER_INVARIANTS)
+        render_invariants_kernel<<<grid_for(n, 256), 256, 0, s>>>(v, ctx->opt.precision, first_ray, n, (double *)out);
+    else
+        render_pixels_kernel<<<grid_for(n, 256), 256, 0, s>>>(v, ctx->opt.precision, first_ray, n, kind, out);
     return check_launch();
 }
 
