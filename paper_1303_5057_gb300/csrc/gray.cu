@@ -2890,8 +2890,8 @@ int gray_shadow(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_
     if (cudaMemsetAsync(out, 0, sizeof(gray_shadow_info) * (size_t)n_images, s) != cudaSuccess)
         return GRAY_ECUDA;
     StateView v = make_view((void *)state, n_state, ctx->opt.precision);
-    shadow_accum_kernel<<<grid_for(total, 256), 256, 0, s>>>(v, first_ray, (const ImageDev *)dimg, n_images, total,
-                                                            out);
+    shadow_accum_kernel<<<grid_for(total, SHADOW_RAYS), SHADOW_BLOCK, 0, s>>>(v, first_ray, (const ImageDev *)dimg,
+                                                                             n_images, total, out);
     if ((rc = check_launch()))
         return rc;
     shadow_final_kernel<<<grid_for(n_images, 128), 128, 0, s>>>((const ImageDev *)dimg, n_images, out);
