@@ -1747,27 +1747,62 @@ __global__ void __launch_bounds__(RING_BLOCK) ring_rows_kernel(const int4 *S0, i
     }
 }
 
-// Eqs. 6-8 from each image's boundary rows, one thread per image, in a fixed
-// order: extremes of alpha_0 = R_b cos(vartheta), centre, then trapezoidal
-// means over the rows' angles of R and of (R - <R>)^2.
-__global__ void ring_final_kernel(const RingDev *imgs, int n_images, const double *boundary, gray_ring_info *out)
+// Sum over the block of each thread's value, in a fixed order (shuffles
+// within the warp, then the warps in order): every thread gets the total.
+__device__ double ring_block_sum(double x, double *part)
 {
-    const int k = blockIdx.x * blockDim.x + threadIdx.x;
-    if (k >= n_images)
-        return;
-    const RingDev im = imgs[k];
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1)
+        x += __shfl_xor_sync(0xffffffffu, x, off);
+    if ((threadIdx.x & 31) == 0)
+        part[threadIdx.x >> 5] = x;
+    __syncthreads();
+    double t = 0.0;
+    for (int w = 0; w < RING_BLOCK / 32; ++w)
+        t += part[w];
+    __syncthreads();
+    return t;
+}
+
+// Eqs. 6-8 from each image's boundary rows, one block per image, in a fixed
+// order: extremes of alpha_0 = R_b cos(vartheta), centre, then trapezoidal
+// means over the rows' angles of R and of (R - <R>)^2.  Each row's sine,
+// cosine and square root run on the FP64 pipe, which takes an instruction of
+// one warp every 64 cycles whatever its lanes: one thread per image walked
+// its 181 rows three times in 666 us; a thread per row takes 14 us.
+__global__ void __launch_bounds__(RING_BLOCK) ring_final_kernel(const RingDev *imgs, const double *boundary,
+                                                                gray_ring_info *out)
+{
+    __shared__ double part[RING_BLOCK / 32], s_min[RING_BLOCK / 32], s_max[RING_BLOCK / 32];
+    const RingDev im = imgs[blockIdx.x];
     const double *Rb = boundary + im.first_row;
-    double a_min = 0.0, a_max = 0.0;
-    for (int j = 0; j < im.ny; ++j) {
+    const int tid = threadIdx.x;
+    double a_min = INFINITY, a_max = -INFINITY;
+    for (int j = tid; j < im.ny; j += RING_BLOCK) {
         double sn, cs;
         sincos(im.th0 + (double)j * im.dth, &sn, &cs);
         const double al = Rb[j] * cs;
-        a_min = (j == 0 || al < a_min) ? al : a_min;
-        a_max = (j == 0 || al > a_max) ? al : a_max;
+        a_min = al < a_min ? al : a_min;
+        a_max = al > a_max ? al : a_max;
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        const double lo = __shfl_xor_sync(0xffffffffu, a_min, off), hi = __shfl_xor_sync(0xffffffffu, a_max, off);
+        a_min = lo < a_min ? lo : a_min;
+        a_max = hi > a_max ? hi : a_max;
+    }
+    if ((tid & 31) == 0) {
+        s_min[tid >> 5] = a_min;
+        s_max[tid >> 5] = a_max;
+    }
+    __syncthreads();
+    for (int w = 0; w < RING_BLOCK / 32; ++w) {
+        a_min = s_min[w] < a_min ? s_min[w] : a_min;
+        a_max = s_max[w] > a_max ? s_max[w] : a_max;
     }
     const double c = 0.5 * (a_min + a_max);
     double sum = 0.0, wsum = 0.0;
-    for (int j = 0; j < im.ny; ++j) {
+    for (int j = tid; j < im.ny; j += RING_BLOCK) {
         double sn, cs;
         sincos(im.th0 + (double)j * im.dth, &sn, &cs);
         const double R = sqrt((Rb[j] * cs - c) * (Rb[j] * cs - c) + (Rb[j] * sn) * (Rb[j] * sn));
@@ -1775,22 +1810,26 @@ __global__ void ring_final_kernel(const RingDev *imgs, int n_images, const doubl
         sum += w * R;
         wsum += w;
     }
-    const double R_mean = sum / wsum;
+    wsum = ring_block_sum(wsum, part);
+    const double R_mean = ring_block_sum(sum, part) / wsum;
     double var = 0.0;
-    for (int j = 0; j < im.ny; ++j) {
+    for (int j = tid; j < im.ny; j += RING_BLOCK) {
         double sn, cs;
         sincos(im.th0 + (double)j * im.dth, &sn, &cs);
         const double R = sqrt((Rb[j] * cs - c) * (Rb[j] * cs - c) + (Rb[j] * sn) * (Rb[j] * sn));
         const double w = (im.ny > 1 && (j == 0 || j == im.ny - 1)) ? 0.5 : 1.0;
         var += w * (R - R_mean) * (R - R_mean);
     }
-    gray_ring_info *o = out + k;
-    o->D = fabs(c);
-    o->R_mean = R_mean;
-    o->A = 2.0 * sqrt(var / wsum);
-    o->alpha_min = a_min;
-    o->alpha_max = a_max;
-    o->n_rows = im.ny;
+    var = ring_block_sum(var, part);
+    if (tid == 0) {
+        gray_ring_info *o = out + blockIdx.x;
+        o->D = fabs(c);
+        o->R_mean = R_mean;
+        o->A = 2.0 * sqrt(var / wsum);
+        o->alpha_min = a_min;
+        o->alpha_max = a_max;
+        o->n_rows = im.ny;
+    }
 }
 
 // --------------------------------------------------------------------------
@@ -2953,7 +2992,7 @@ int gray_ring(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_st
     ring_rows_kernel<<<(unsigned)rows, RING_BLOCK, 0, s>>>(v.S0, first_ray, dimg, n_images, rb, out);
     rc = check_launch();
     if (!rc) {
-        ring_final_kernel<<<grid_for(n_images, 128), 128, 0, s>>>(dimg, n_images, rb, out);
+        ring_final_kernel<<<(unsigned)n_images, RING_BLOCK, 0, s>>>(dimg, rb, out);
         rc = check_launch();
     }
     cudaError_t e = cudaFreeAsync(dmem, s);
