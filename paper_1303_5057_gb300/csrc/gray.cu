@@ -4,6 +4,7 @@
 //   setup_images_kernel / setup_rays_kernel  image-plane initial conditions (double)
 //   trace32_kernel<MODE>, trace64_kernel     persistent backward RK4 tracers
 //                                            (single precision, double)
+//   trace64_quad_kernel                      double precision with four lanes per ray
 //   zone_kernel<RETURN, T>                   the near-horizon zone of the
 //                                            selective mode (double-single or double)
 //   probe_rays_kernel, plan_*_kernel         the longest-first planner
@@ -24,9 +25,11 @@
 // its lanes are idle, so every launch ends.
 #include "gray.h"
 #include "kerr.cuh"
+#include "quad.cuh"
 
 #include <cuda_runtime.h>
 
+#include <algorithm>
 #include <atomic>
 #include <cmath>
 #include <type_traits>
@@ -573,6 +576,7 @@ struct TraceArgs {
                           // S1.y == epoch means S1.z counts this call's steps
     int one_per_thread; // the paper's launch: thread g takes queue slot g only
     int stop_equator;   // Sec. 3 grid projection: stop at the equatorial plane
+    int64_t handover;   // double-precision pass: the last `handover` rays of the queue go to the hand-off list
     int zone_return;    // zone pass: a ray climbing out of the zone goes to the return list
     double h_frac, h_min, eps_xi, cap_frac, r_esc_frac, r_sw;
     Workspace *ws;
@@ -813,8 +817,12 @@ template <int MODE, int MAXREG = 128> __global__ void __maxnreg__(MAXREG) trace3
     warp_stats<float>(A, lane, tot_steps, tot_euler, 0ull);
 }
 
-// Double-precision persistent tracer over every ray of a GRAY_FP64 buffer.
-__global__ void __launch_bounds__(128) trace64_kernel(TraceArgs A)
+// Double-precision persistent tracer over every ray of a GRAY_FP64 buffer, one
+// ray per lane.  With A.handover the warps count the rays they finish; once
+// the queue is empty and no more than A.handover rays are left on the whole
+// chip, every warp stores its rays as they stand and lists them for the
+// four-lane kernel, which steps a lone ray 1.5 times faster.
+__global__ void __launch_bounds__(32) trace64_kernel(TraceArgs A)
 {
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
@@ -839,10 +847,23 @@ __global__ void __launch_bounds__(128) trace64_kernel(TraceArgs A)
     for (int m = 0; m < 8; ++m)
         cz[m] = 0.0;
 
+    unsigned resolved = 0; // queue slots this lane has finished with since its last report
+    bool give = false;     // the rays left go to the hand-off list
     for (;;) {
         const bool stop = cancelled(A, lane); // gray_cancel, as in trace32_kernel
         if (stop)
             exhausted = true;
+        if (A.handover > 0 && !stop) {
+            const unsigned r = __reduce_add_sync(FULL, resolved);
+            resolved = 0;
+            long long left = 0;
+            if (lane == 0) {
+                if (r)
+                    atomicAdd(&A.ws->demoted, (unsigned long long)r);
+                left = nq - (long long)*(volatile unsigned long long *)&A.ws->demoted;
+            }
+            give = exhausted && __shfl_sync(FULL, left, 0) <= A.handover;
+        }
         while (!exhausted) {
             const unsigned idle = __ballot_sync(FULL, !has);
             if (idle == 0)
@@ -856,11 +877,13 @@ __global__ void __launch_bounds__(128) trace64_kernel(TraceArgs A)
             if (!has) {
                 const int64_t slot = (int64_t)base + __popc(idle & ((1u << lane) - 1u));
                 const int64_t my = slot < nq ? queue_ray(A, slot) : -1;
+                resolved += slot < nq; // taken back if the slot holds a ray to trace
                 if (my >= 0) {
                     const int4 s0 = v.S0[my];
                     if (s0.x == GRAY_RAY_ACTIVE) {
                         const int4 s1 = v.S1[my];
                         has = true;
+                        --resolved;
                         id = my;
                         steps = s0.y;
                         euler = s0.z;
@@ -881,6 +904,19 @@ __global__ void __launch_bounds__(128) trace64_kernel(TraceArgs A)
         }
         if (!__any_sync(FULL, has))
             break;
+
+        if (give) {
+            int rank;
+            const unsigned long long hb = warp_count(&A.ws->handoff, has, lane, &rank);
+            if (has) {
+                v.L[hb + rank] = (int)id;
+                st_d4(v.X, id, y[0], y[1], y[2], y[3]);
+                st_d4(v.K, id, y[4], y[5], y[6], y[7]);
+                v.S0[id] = make_int4(GRAY_RAY_ACTIVE, steps, euler, remaps);
+                v.S1[id] = make_int4(n64, epoch, used, 0);
+            }
+            break;
+        }
 
         for (int k = 0; k < A.refill; ++k) {
             if (has) {
@@ -908,7 +944,146 @@ __global__ void __launch_bounds__(128) trace64_kernel(TraceArgs A)
                     v.S0[id] = make_int4(status, steps, euler, remaps);
                     v.S1[id] = make_int4(n64, epoch, used, 0);
                     has = false;
+                    ++resolved;
                 }
+            }
+        }
+    }
+    warp_stats<double>(A, lane, tot_steps, tot_euler, 0ull);
+}
+
+// Double-precision tracer with four lanes per ray (quad.cuh), for queues too
+// short to fill the chip with one ray per lane: eight rays to a warp, the
+// lanes of a quad sharing every load, count and decision.  Same queue, refill,
+// budget and cancel rules as trace64_kernel, and the same bits per ray.
+__global__ void __launch_bounds__(32) trace64_quad_kernel(TraceArgs A)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, m = lane & 3;
+    const StateView &v = A.v;
+    StepOpt<double> O;
+    O.h_frac = A.h_frac;
+    O.h_min = A.h_min;
+    O.eps_xi = A.eps_xi;
+    O.step_rule = A.step_rule;
+    O.stop_equator = A.stop_equator;
+
+    // idle quads step a photon at rest: finite, no rare path
+    bool has = false, exhausted = false;
+    int64_t id = 0;
+    double x = m == 1 ? 10.0 : 1.0, k = 0.0, fin[4];
+    Hole<double> H = make_hole(0.0, 0.0, 1000.0, 1.0, 1.0, 0.0);
+    const Geo<double> idle_geo{10.0, 1.0, 0.0, 100.0, 80.0, 0.01, 0.0125, 1.0};
+    Geo<double> geo = idle_geo;
+    QuadPre pre{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
+    bool fresh = false; // the quad's ray was just loaded: its geometry is not formed yet
+    int steps = 0, euler = 0, remaps = 0, n64 = 0, used = 0;
+    unsigned long long tot_steps = 0, tot_euler = 0; // lane 0 of the quad counts
+    const int64_t nq = queue_length(A);
+    const int epoch = *A.epoch_dev;
+
+    for (;;) {
+        const bool stop = cancelled(A, lane); // gray_cancel, as in trace32_kernel
+        if (stop)
+            exhausted = true;
+        while (!exhausted) {
+            const unsigned idle = __ballot_sync(FULL, !has) & 0x11111111u; // a bit per quad
+            if (idle == 0)
+                break;
+            const int cnt = __popc(idle);
+            const int leader = __ffs(idle) - 1;
+            unsigned long long base = 0;
+            if (lane == leader)
+                base = atomicAdd(&A.ws->head, (unsigned long long)cnt);
+            base = __shfl_sync(FULL, base, leader);
+            if (!has) {
+                const int64_t slot = (int64_t)base + __popc(idle & ((1u << (lane & 28)) - 1u));
+                const int64_t my = slot < nq ? queue_ray(A, slot) : -1;
+                if (my >= 0) {
+                    const int4 s0 = v.S0[my];
+                    if (s0.x == GRAY_RAY_ACTIVE) {
+                        const int4 s1 = v.S1[my];
+                        has = fresh = true;
+                        id = my;
+                        steps = s0.y;
+                        euler = s0.z;
+                        remaps = s0.w;
+                        n64 = s1.x;
+                        used = (s1.y == epoch) ? s1.z : 0;
+                        const d4 p = ld_d4(v.P, my);
+                        H = make_hole(p.x, p.y, p.z, A.cap_frac, A.r_esc_frac, A.r_sw);
+                        x = ((const double *)v.X)[4 * my + m];
+                        k = ((const double *)v.K)[4 * my + m];
+                    }
+                }
+            }
+            if ((int64_t)base + cnt >= nq)
+                exhausted = true;
+        }
+        if (!__any_sync(FULL, has))
+            break;
+        if (__any_sync(FULL, fresh)) {
+            double s, c;
+            sincos(qget(x, 2), &s, &c);
+            Geo<double> gn;
+            QuadPre qn;
+            quad_point<false>(H, m, qget(x, 1), 0.0, 0.0, 1.0, true, false, s, c, qget(k, 0), qget(k, 1), qget(k, 2),
+                              qget(k, 3), gn, qn);
+            if (fresh) {
+                geo = gn;
+                pre = qn;
+            }
+            fresh = false;
+        }
+
+        for (int b = 0; b < A.refill; ++b) {
+            int status = GRAY_RAY_ACTIVE;
+            bool yield = false;
+            const double r0 = x; // lane m's position, the stop point of a capped ray
+            bool live = has;
+            if (has && steps >= A.max_steps) {
+                status = GRAY_RAY_STEP_CAP;
+                live = false;
+            } else if (has && (stop || (A.budget > 0 && used >= A.budget))) {
+                yield = true;
+                live = false;
+            }
+            const double xb = x, kb = k;
+            const Geo<double> gb = geo;
+            const QuadPre qb = pre;
+            const QuadStep q = quad_step<GRAY_RAY_CAPTURED, GRAY_RAY_ESCAPED, GRAY_RAY_NONFINITE, GRAY_RAY_EQUATOR>(
+                H, O, m, live, x, k, geo, pre, fin);
+            if (live) {
+                status = q.status;
+                euler += q.redo;
+                remaps += q.remap;
+                ++steps;
+                ++used;
+                if (m == 0) {
+                    ++tot_steps;
+                    tot_euler += q.redo;
+                }
+            } else {
+                x = xb;
+                k = kb;
+                geo = gb;
+                pre = qb;
+            }
+            if (has && (status != GRAY_RAY_ACTIVE || yield)) {
+                ((double *)v.X)[4 * id + m] = x;
+                ((double *)v.K)[4 * id + m] = k;
+                if (status != GRAY_RAY_ACTIVE)
+                    ((double *)v.F)[4 * id + m] =
+                        status == GRAY_RAY_STEP_CAP ? r0 : qsel(m, fin[0], fin[1], fin[2], fin[3]);
+                if (m == 0) {
+                    v.S0[id] = make_int4(status, steps, euler, remaps);
+                    v.S1[id] = make_int4(n64, epoch, used, 0);
+                }
+                has = false;
+                x = m == 1 ? 10.0 : 1.0;
+                k = 0.0;
+                geo = idle_geo;
+                pre = QuadPre{0.0, 0.0, 0.0, 0.0, 0.0, 0.0};
             }
         }
     }
@@ -2415,6 +2590,7 @@ TraceArgs make_trace_args(gray_ctx *ctx, void *state, int64_t n_state, int64_t s
     A.cancel = (const int *)&ctx->aux[AUX_CANCEL];
     A.one_per_thread = o.launch == GRAY_LAUNCH_ONE_PER_THREAD;
     A.stop_equator = o.stop_equator;
+    A.handover = 0;
     A.zone_return = 0;
     return A;
 }
@@ -2448,6 +2624,46 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
         trace32_kernel<MODE><<<persistent_grid(ctx, (const void *)trace32_kernel<MODE>, block, work), block, 0, s>>>(A);
 }
 
+// A double-precision pass.  An SM takes one FP64 instruction per 19 cycles and
+// a warp at most one per 64, so four warps fill the pipe; more only slow each
+// other down, and the longest rays with them.  Warps are single blocks, spread
+// evenly over the SMs, W64_PER_SM = 5 to an SM.  (300 x 211 image, a = 0.9,
+// i = 75 deg, planned: three 128-thread blocks per SM 107 ms, 4 / 5 / 6 / 8
+// warps 60 / 66 / 74 / 90 ms; 512^2: 136 ms, then 109 / 108 / 108 / 115;
+// 1024 x 640: 253 ms, then 251 / 250 / 250 / 250.)
+//
+// Up to QUAD_RAYS_PER_SM rays per SM go to the four-lane kernel at once: there
+// a step of one ray takes 12.7 us instead of 19 (64^2: 45 -> 29 ms; 128^2
+// planned: 60 -> 42), while a chip full of rays does 1.7 times the steps per
+// second with a ray per lane (1024 x 640: 250 ms against 433; 300 x 211
+// planned is the crossover: 60 against 51 ms, under Eq. 2 48 against 70).  In
+// longer queues the one-lane kernel hands its last rays over (A.handover;
+// 300 x 211: 66 -> 54 ms planned, 62 -> 51 in natural order, 48 -> 44 Eq. 2).
+constexpr int W64_PER_SM = 5, QUAD_PER_SM = 6, QUAD_RAYS_PER_SM = 160, QUAD_HANDOVER_PER_SM = 32;
+
+int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
+{
+    const int64_t sms = ctx->num_sms;
+    int64_t per_sm = ctx->opt.blocks_per_sm > 0 ? 4 * (int64_t)ctx->opt.blocks_per_sm : W64_PER_SM;
+    int64_t quad_work = work;
+    if (work > QUAD_RAYS_PER_SM * sms) {
+        A.handover = std::min(QUAD_HANDOVER_PER_SM * sms, A.n); // the list holds n entries
+        trace64_kernel<<<(unsigned)std::min(per_sm * sms, (work + 31) / 32), 32, 0, s>>>(A);
+        const int rc = check_launch();
+        if (rc)
+            return rc;
+        A.handover = 0;
+        A.order = A.v.L;
+        A.n_queue_dev = &ctx->ws->handoff;
+        quad_work = QUAD_HANDOVER_PER_SM * sms; // at most; the kernel reads the list's length
+        if (cudaMemsetAsync(&ctx->ws->head, 0, sizeof(unsigned long long), s) != cudaSuccess)
+            return GRAY_ECUDA;
+    }
+    per_sm = ctx->opt.blocks_per_sm > 0 ? per_sm : QUAD_PER_SM;
+    trace64_quad_kernel<<<(unsigned)std::min(per_sm * sms, (quad_work + 7) / 8), 32, 0, s>>>(A);
+    return check_launch();
+}
+
 // probe: the planner's probe pass (the uncapped instantiation).
 int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s, bool probe = false)
 {
@@ -2472,10 +2688,7 @@ int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s,
     const int block = ctx->opt.block > 0 ? ctx->opt.block : 128;
     switch (ctx->opt.precision) {
     case GRAY_FP64:
-        // the double kernels are built for 128-thread blocks (their launch
-        // bounds); the tunable block size is the single-precision pass's
-        trace64_kernel<<<persistent_grid(ctx, (const void *)trace64_kernel, 128, work), 128, 0, s>>>(A);
-        break;
+        return launch_trace64(ctx, A, work, s);
     case GRAY_FP32:
         launch_trace32<GRAY_FP32>(ctx, A, work, block, probe, s);
         break;

@@ -1,0 +1,73 @@
+"""Double precision with four lanes per ray against one ray per lane.
+
+Queues of up to 160 rays per SM are traced by the four-lane kernel, longer ones
+by the one-lane kernel, whose last rays the four-lane kernel takes over.  Both
+do the same operations on the same operands, so a ray's record is the same
+bits in each (no tolerance): an image alone, and as many copies of it in one
+buffer as pass the limit."""
+import math
+
+import numpy as np
+import pytest
+import torch
+
+from paper_1303_5057_gb300 import gray
+from paper_1303_5057_gb300 import inputs as I
+
+pytestmark = pytest.mark.gpu
+
+CASES = {
+    # fewer rays than a warp's eight quads, one more, an odd number of warps
+    "1": (I.Image(a=0.9, incl=1.0, nx=1, ny=1, alpha0=3.0, alpha1=4.0, beta0=1.0, beta1=2.0), {}),
+    "7": (I.Image(a=0.9, incl=1.0, nx=7, ny=1), {}),
+    "9": (I.Image(a=0.9, incl=1.0, nx=3, ny=3), {}),
+    # pole crossings, Euler redos, far stage angles, both stop surfaces
+    "kerr": (I.Image(a=0.99, incl=math.radians(90.0), nx=37, ny=23), {}),
+    "face_on_eq2": (I.Image(a=0.998, incl=math.radians(12.0), nx=29, ny=17), {"step_rule": gray.STEP_EQ2}),
+    "equator": (I.Image(a=0.95, incl=math.radians(60.0), nx=30, ny=21, alpha0=-15, alpha1=15, beta0=-15, beta1=15),
+                {"stop_equator": 1}),
+    "flat": (I.Image(a=0.3, M=0.0, incl=1.0, nx=16, ny=9), {}),
+    "retrograde": (I.Image(a=-0.7, incl=math.radians(120.0), nx=19, ny=18), {}),
+    "step_cap": (I.Image(a=0.9, incl=1.2, nx=17, ny=16), {"max_steps": 211}),
+}
+
+
+def records(images, opt, budgets):
+    tr = gray.Tracer(opt, sum(im.n for im in images))
+    tr.setup(images)
+    for b in budgets:
+        tr.trace(step_budget=b)
+    rec = tr.records()
+    tr.close()
+    return rec
+
+
+@pytest.mark.parametrize("budgets", [(0,), (5, 1, 200, 0)], ids=["whole", "split"])
+@pytest.mark.parametrize("name", CASES)
+def test_four_lanes_per_ray_give_the_bits_of_one(name, budgets):
+    im, options = CASES[name]
+    opt = gray.Options(precision=gray.FP64, **{"max_steps": 20000, **options})
+    alone = records([im], opt, budgets)
+    limit = 160 * torch.cuda.get_device_properties(0).multi_processor_count
+    copies = limit // im.n + 1
+    many = records([im] * copies, opt, budgets).reshape(copies, im.n, -1)
+    assert np.all(alone[:, 0] != gray.ACTIVE)
+    same = (many == alone[None]) | (np.isnan(many) & np.isnan(alone[None]))
+    assert np.all(same), np.argwhere(~same)[:5]
+
+
+def test_a_short_state_with_a_long_queue_keeps_its_hand_off_list():
+    """A queue longer than the four-lane limit over a state of fewer rays (its
+    surplus entries lie outside the buffer and are skipped)."""
+    im = I.Image(a=0.9, incl=1.0, nx=9, ny=7)
+    opt = gray.Options(precision=gray.FP64, max_steps=20000)
+    want = records([im], opt, (0,))
+    limit = 160 * torch.cuda.get_device_properties(0).multi_processor_count
+    order = torch.full((limit + 100,), -1, dtype=torch.int32, device="cuda")
+    order[50:50 + im.n] = torch.arange(im.n, dtype=torch.int32, device="cuda")
+    tr = gray.Tracer(opt, im.n)
+    tr.setup([im])
+    rc, n_active, _ = tr.trace(order=order)
+    rec = tr.records()
+    tr.close()
+    assert rc == 0 and n_active == 0 and np.array_equal(rec, want)
