@@ -388,7 +388,7 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
     T h = step_size(H, O, y);
     T a1[4];
     accel_geo(H, g, y[4], y[5], y[6], y[7], a1);
-    const T hh = T(0.5) * h;
+    const T hh = scaled(h, 0.5);
     const T dr = KAHAN ? -c[1] : T(0), dth = KAHAN ? -c[2] : T(0);
     const T h6 = sixth(h);
     T inc[8];
@@ -408,7 +408,7 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
 #pragma unroll 1
         for (int stage = 0; stage < 3; ++stage) {
             const T cs = stage < 2 ? hh : h;
-            const T w = stage < 2 ? T(2) : T(1);
+            const float w = stage < 2 ? 2.0f : 1.0f;
             const T rs = fma(cs, pk[1], y[1]), ths = fma(cs, pk[2], y[2]);
             T ks[4], as[4];
 #pragma unroll
@@ -417,8 +417,8 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
             accel_geo(H, geometry_rel(H, g, rs, cs * pk[2], ths, dr, dth), ks[0], ks[1], ks[2], ks[3], as);
 #pragma unroll
             for (int m = 0; m < 4; ++m) {
-                sk[m] = fma(w, ks[m], sk[m]);
-                sa[m] = fma(w, as[m], sa[m]);
+                sk[m] = fma_scaled(ks[m], w, sk[m]);
+                sa[m] = fma_scaled(as[m], w, sa[m]);
                 pk[m] = ks[m];
                 pa[m] = as[m];
             }
@@ -1113,6 +1113,31 @@ template <> struct ZoneArith<ds> {
     static __device__ __forceinline__ float to_float(ds v) { return v.hi; }
 };
 
+// The state of a ray of the hand-off list in the zone's arithmetic.
+template <typename T> __device__ __forceinline__ void load_zone_state(const StateView &v, int64_t my, int flags, T *y)
+{
+    using Z = ZoneArith<T>;
+    if (flags & FLAG_DOUBLE_REPR) {
+        // exact double state parked in the four single planes (IEEE-double zone)
+        const double2 q0 = ((const double2 *)v.X)[my], q1 = ((const double2 *)v.K)[my];
+        const double2 q2 = ((const double2 *)v.CX)[my], q3 = ((const double2 *)v.CK)[my];
+        const double q[8] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y};
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            float hi, c;
+            ZoneArith<double>::to_pair(q[m], hi, c);
+            y[m] = std::is_same<T, ds>::value ? Z::from_pair(hi, c) : T(q[m]);
+        }
+    } else {
+        const float4 X = ld_f4(v.X, my), K = ld_f4(v.K, my);
+        const float4 CX = ld_f4(v.CX, my), CK = ld_f4(v.CK, my);
+        y[0] = Z::from_pair(X.x, CX.x); y[1] = Z::from_pair(X.y, CX.y);
+        y[2] = Z::from_pair(X.z, CX.z); y[3] = Z::from_pair(X.w, CX.w);
+        y[4] = Z::from_pair(K.x, CK.x); y[5] = Z::from_pair(K.y, CK.y);
+        y[6] = Z::from_pair(K.z, CK.z); y[7] = Z::from_pair(K.w, CK.w);
+    }
+}
+
 // Zone kernel of GRAY_FP32_KAHAN_SEL64: the rays of the hand-off list, in
 // extended precision T (double, or double-single on the single-precision
 // pipe: GRAY_ZONE_DS) while r < r_demote (= r_promote + r_sw).  RETURN = true
@@ -1203,25 +1228,7 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
                             Hf = make_hole_f(v.PF0[my], v.PF1[my], (float)A.cap_frac, (float)A.r_esc_frac,
                                              (float)A.r_sw);
                         r_demote = Hd.r_promote + r_sw;
-                        if (s1.w & FLAG_DOUBLE_REPR) {
-                            // exact double state parked in the four single planes (IEEE-double zone)
-                            const double2 q0 = ((const double2 *)v.X)[my], q1 = ((const double2 *)v.K)[my];
-                            const double2 q2 = ((const double2 *)v.CX)[my], q3 = ((const double2 *)v.CK)[my];
-                            const double q[8] = {q0.x, q0.y, q1.x, q1.y, q2.x, q2.y, q3.x, q3.y};
-#pragma unroll
-                            for (int m = 0; m < 8; ++m) {
-                                float hi, c;
-                                ZoneArith<double>::to_pair(q[m], hi, c);
-                                yd[m] = std::is_same<T, ds>::value ? Z::from_pair(hi, c) : T(q[m]);
-                            }
-                        } else {
-                            const float4 X = ld_f4(v.X, my), K = ld_f4(v.K, my);
-                            const float4 CX = ld_f4(v.CX, my), CK = ld_f4(v.CK, my);
-                            yd[0] = Z::from_pair(X.x, CX.x); yd[1] = Z::from_pair(X.y, CX.y);
-                            yd[2] = Z::from_pair(X.z, CX.z); yd[3] = Z::from_pair(X.w, CX.w);
-                            yd[4] = Z::from_pair(K.x, CK.x); yd[5] = Z::from_pair(K.y, CK.y);
-                            yd[6] = Z::from_pair(K.z, CK.z); yd[7] = Z::from_pair(K.w, CK.w);
-                        }
+                        load_zone_state(v, my, s1.w, yd);
                         gd = geometry(Hd, yd[1], yd[2]);
                     }
                 }

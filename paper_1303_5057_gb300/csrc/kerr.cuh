@@ -39,6 +39,7 @@
 
 #include <cuda_runtime.h>
 #include <math.h>
+#include <type_traits>
 
 namespace gray {
 
@@ -305,6 +306,12 @@ __device__ __forceinline__ float recip_approx(float x)
 }
 __device__ __forceinline__ double recip_approx(double x) { return recip(x); }
 
+// x k and x k + c for a power of two k: exact scalings, which double-single
+// takes word by word (2 and 13 instructions, where its general product and
+// product-sum take 7 and 15).
+template <typename T> __device__ __forceinline__ T scaled(T x, double k) { return T(k) * x; }
+template <typename T> __device__ __forceinline__ T fma_scaled(T x, double k, T c) { return fma(x, T(k), c); }
+
 // Geometry of one point (r, theta): the quantities every right-hand side and
 // the Eq. 4 monitor need, with the reciprocals of Sigma, Delta and sin(theta).
 template <typename T> struct Geo {
@@ -316,11 +323,12 @@ template <typename T> struct Geo {
 // FMA pipe), each within 2 ulp (unit test); forming the three from one
 // reciprocal of Sigma Delta sin takes eight issue slots and rounds up to
 // five times (single-precision pass 8.33 -> 8.00 ms on the 1024^2 image).
-// Double and double-single keep the one reciprocal (there each reciprocal
-// is a refined sequence).
+// Double-single likewise (14 instructions each, off the chain through Sigma
+// Delta sin).  Double keeps the one reciprocal (there each is a refined
+// sequence on the narrow FP64 pipe).
 template <typename T> __device__ __forceinline__ void geometry_reciprocals(Geo<T> &g)
 {
-    if constexpr (sizeof(T) == 4) {
+    if constexpr (!std::is_same<T, double>::value) {
         g.iS = recip_approx(g.Sigma);
         g.iD = recip_approx(g.Delta);
         g.is = recip_approx(g.s);
@@ -446,10 +454,10 @@ __device__ __forceinline__ void accel_geo(const Hole<T> &H, const Geo<T> &g, T k
 {
     const T r = g.r, iS = g.iS;
     const T r2 = r * r, s2 = g.s * g.s, sc = g.s * g.c;
-    const T A = fma(T(2), r2, -g.Sigma);
+    const T A = fma_scaled(r2, 2.0, -g.Sigma);
     const T P = r2 + H.a2;
     const T V = -(H.t2a * s2) * kp;
-    const T X = fma(V, T(0.5), kt) * iS;
+    const T X = fma_scaled(V, 0.5, kt) * iS;
     const T u = kr * g.iD;
     const T q = kr * u;
     const T krkh = kr * kh, kh2 = kh * kh, kp2 = kp * kp;
@@ -465,12 +473,12 @@ __device__ __forceinline__ void accel_geo(const Hole<T> &H, const Geo<T> &g, T k
     acc[1] = iS * sr;
     // theta
     const T Z = (H.t2Ma * r) * X;
-    const T hth = fma(Z, fma(H.a, X, T(-2) * kp), fma(P, kp2, H.a2 * (kh2 - q)));
-    acc[2] = iS * fma(r * krkh, T(-2), sc * hth);
+    const T hth = fma(Z, fma(H.a, X, scaled(kp, -2.0)), fma(P, kp2, H.a2 * (kh2 - q)));
+    acc[2] = iS * fma_scaled(r * krkh, -2.0, sc * hth);
     // phi
     const T inner = fma(iS, fma(H.m2M * r2, kp, (H.Ma * A) * X), r * kp);
     const T up2 = fma(-Z, iS, kp);
-    acc[3] = T(-2) * fma(u, inner, ((g.c * g.is) * kh) * up2);
+    acc[3] = scaled(fma(u, inner, ((g.c * g.is) * kh) * up2), -2.0);
 }
 
 // Eq. 4 test without its division: |xi + 1| > eps  <=>
@@ -566,6 +574,19 @@ __device__ __forceinline__ ds ds_mul(ds x, ds y)
     e = fmaf(x.lo, y.hi, e);
     return ds_fast(p, e);
 }
+// x y + z with one normalisation: the product's two words enter the sum as
+// they are (15 instructions, 52 cycles of latency, where a product, normalised,
+// and a sum take 18 and 64).  __fmul_rn keeps the compiler from contracting
+// the exact product word into the sum.
+__device__ __forceinline__ ds ds_fma(ds x, ds y, ds z)
+{
+    const float p = __fmul_rn(x.hi, y.hi);
+    float e = fmaf(x.hi, y.hi, -p);
+    e = fmaf(x.hi, y.lo, e);
+    e = fmaf(x.lo, y.hi, e);
+    const ds s = ds_two_sum(p, z.hi);
+    return ds_fast(s.hi, s.lo + (e + z.lo));
+}
 __device__ __forceinline__ ds ds_mulf(ds x, float y)
 {
     const float p = x.hi * y;
@@ -603,7 +624,9 @@ __device__ __forceinline__ bool operator<(ds a, ds b) { return a.hi < b.hi || (a
 __device__ __forceinline__ bool operator>(ds a, ds b) { return b < a; }
 __device__ __forceinline__ bool operator<=(ds a, ds b) { return !(b < a) && a.hi == a.hi && b.hi == b.hi; }
 __device__ __forceinline__ bool operator>=(ds a, ds b) { return b <= a; }
-__device__ __forceinline__ ds fma(ds a, ds b, ds c) { return ds_add(ds_mul(a, b), c); }
+__device__ __forceinline__ ds fma(ds a, ds b, ds c) { return ds_fma(a, b, c); }
+__device__ __forceinline__ ds scaled(ds x, double k) { return ds{x.hi * (float)k, x.lo * (float)k}; }
+__device__ __forceinline__ ds fma_scaled(ds x, double k, ds c) { return ds_add(scaled(x, k), c); }
 __device__ __forceinline__ ds fabs(ds a) { return a.hi < 0.0f ? ds_neg(a) : a; }
 __device__ __forceinline__ ds fmin(ds a, ds b) { return b < a ? b : a; }
 __device__ __forceinline__ ds fmax(ds a, ds b) { return a < b ? b : a; }
@@ -720,7 +743,7 @@ __device__ __forceinline__ void geodesic_accel(const Hole<T> &H, T r, T th, T kt
 template <typename T> __device__ __forceinline__ T step_size(const Hole<T> &H, const StepOpt<T> &O, const T *y)
 {
     const T r = y[1], kr = y[5];
-    const T guard = (r - H.r_h) * (T(0.5) * recip(fabs(kr)));
+    const T guard = (r - H.r_h) * scaled(recip(fabs(kr)), 0.5);
     T h;
     if (O.step_rule == 1)
         h = fmin(O.h_frac * recip(fabs(kr) * recip(r) + fabs(y[6]) + fabs(y[7])), guard);
