@@ -173,6 +173,7 @@ struct Workspace {
     unsigned long long handoff; // rays appended to the hand-off list by the current pass
     unsigned long long demoted; // rays returned to single precision by the current zone pass
     unsigned long long zone_steps; // steps taken by the zone kernel in this call
+    unsigned long long front, back; // lead-first queue: rays at its two ends
     unsigned long long cancel;     // the cancel flag as the call ended (copied in by gray_trace)
 };
 
@@ -574,6 +575,7 @@ struct TraceArgs {
     int step_rule;
     const int *epoch_dev; // call counter on the device (bumped by every gray_trace / gray_plan):
                           // S1.y == epoch means S1.z counts this call's steps
+    int split;          // `order` is a lead-first queue (order_rays_kernel): ws->front + ws->back rays
     int one_per_thread; // the paper's launch: thread g takes queue slot g only
     int stop_equator;   // Sec. 3 grid projection: stop at the equatorial plane
     int64_t handover;   // double-precision pass: the last `handover` rays of the queue go to the hand-off list
@@ -594,12 +596,17 @@ __device__ __forceinline__ int64_t queue_length(const TraceArgs &A)
 {
     if (A.n_queue_dev)
         return (int64_t)*(volatile const unsigned long long *)A.n_queue_dev;
+    if (A.split)
+        return (int64_t)(*(volatile const unsigned long long *)&A.ws->front +
+                         *(volatile const unsigned long long *)&A.ws->back);
     return A.order ? A.n_queue : A.n;
 }
-__device__ __forceinline__ int64_t queue_ray(const TraceArgs &A, int64_t slot)
+__device__ __forceinline__ int64_t queue_ray(const TraceArgs &A, int64_t slot, int64_t nq)
 {
     if (!A.order)
         return slot;
+    if (A.split && slot >= (int64_t)*(volatile const unsigned long long *)&A.ws->front)
+        slot += A.n - nq; // the second class ends at the list's end
     const int64_t my = (int64_t)A.order[slot];
     return (my >= 0 && my < A.n) ? my : -1;
 }
@@ -719,7 +726,7 @@ template <int MODE, int MAXREG = 128> __global__ void __maxnreg__(MAXREG) trace3
                 const int64_t slot = A.one_per_thread
                                          ? (int64_t)blockIdx.x * blockDim.x + threadIdx.x
                                          : (int64_t)base + __popc(idle & ((1u << lane) - 1u));
-                const int64_t my = slot < nq ? queue_ray(A, slot) : -1;
+                const int64_t my = slot < nq ? queue_ray(A, slot, nq) : -1;
                 if (my >= 0) {
                     const int4 s0 = v.S0[my];
                     if (s0.x == GRAY_RAY_ACTIVE) {
@@ -876,7 +883,7 @@ __global__ void __launch_bounds__(32) trace64_kernel(TraceArgs A)
             base = __shfl_sync(FULL, base, leader);
             if (!has) {
                 const int64_t slot = (int64_t)base + __popc(idle & ((1u << lane) - 1u));
-                const int64_t my = slot < nq ? queue_ray(A, slot) : -1;
+                const int64_t my = slot < nq ? queue_ray(A, slot, nq) : -1;
                 resolved += slot < nq; // taken back if the slot holds a ray to trace
                 if (my >= 0) {
                     const int4 s0 = v.S0[my];
@@ -998,7 +1005,7 @@ __global__ void __launch_bounds__(32) trace64_quad_kernel(TraceArgs A)
             base = __shfl_sync(FULL, base, leader);
             if (!has) {
                 const int64_t slot = (int64_t)base + __popc(idle & ((1u << (lane & 28)) - 1u));
-                const int64_t my = slot < nq ? queue_ray(A, slot) : -1;
+                const int64_t my = slot < nq ? queue_ray(A, slot, nq) : -1;
                 if (my >= 0) {
                     const int4 s0 = v.S0[my];
                     if (s0.x == GRAY_RAY_ACTIVE) {
@@ -1343,6 +1350,72 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
         }
     }
     warp_stats<double>(A, lane, tot_steps, tot_euler, tot_fp64, true);
+}
+
+// The queue of a trace without a caller's order: the ACTIVE rays, those that
+// will pass close to a pole first.  A persistent pass ends with its last long
+// ray, and under the benchmark step rule the long rays (up to ~3700 steps
+// against a median of 330) are the ones that crawl past a pole: 99 % of the
+// mixed stream's rays over 800 steps have |L_z| < 0.78 M, as 21 % of all have.
+// L_z is conserved, so the state at hand gives it; single precision is enough
+// to sort by.  Rays under 0.7 M fill the list from the front, the others from
+// the back, neighbours staying together (one pair of atomics per block).
+// 524288 mixed rays: pass 8.54 -> 7.10 ms (the bulk alone is ~6 ms at this
+// share of Euler redos); the kernel itself, 16 B of status and 48 B of state
+// per active ray, 10 us.
+constexpr int ORDER_BLOCK = 256, ORDER_RAYS = 1024;
+__global__ void __launch_bounds__(ORDER_BLOCK) order_rays_kernel(StateView v, int64_t n, int *list, Workspace *ws)
+{
+    __shared__ int cnt[2][ORDER_BLOCK / 32];
+    __shared__ unsigned long long base[2];
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const unsigned below = (1u << lane) - 1u;
+    unsigned bits[2][ORDER_RAYS / ORDER_BLOCK];
+    int mine[2] = {0, 0}; // the warp's rays of each class so far
+    const int64_t b0 = (int64_t)blockIdx.x * ORDER_RAYS + warp * (ORDER_RAYS / (ORDER_BLOCK / 32));
+#pragma unroll
+    for (int j = 0; j < ORDER_RAYS / ORDER_BLOCK; ++j) {
+        const int64_t i = b0 + 32 * j + lane;
+        bool active = false, lead = false;
+        if (i < n && v.S0[i].x == GRAY_RAY_ACTIVE) {
+            active = true;
+            const float4 X = ld_f4(v.X, i), K = ld_f4(v.K, i), c = v.PF0[i]; // c: a, M, ..
+            float s, co;
+            fsincos(X.z, &s, &co);
+            const float s2 = s * s, iS = recip_approx(fmaf(c.x * c.x, co * co, X.y * X.y));
+            const float gtp = -2.0f * c.y * X.y * c.x * s2 * iS;
+            const float gpp = s2 * (fmaf(X.y, X.y, c.x * c.x) - c.x * gtp);
+            lead = fabsf(fmaf(gpp, K.w, gtp * K.x)) < 0.7f * c.y;
+        }
+        bits[0][j] = __ballot_sync(0xffffffffu, active && lead);
+        bits[1][j] = __ballot_sync(0xffffffffu, active && !lead);
+        mine[0] += __popc(bits[0][j]);
+        mine[1] += __popc(bits[1][j]);
+    }
+    if (lane < 2)
+        cnt[lane][warp] = mine[lane];
+    __syncthreads();
+    if (tid < 2) {
+        int t = 0;
+        for (int w = 0; w < ORDER_BLOCK / 32; ++w) {
+            const int k = cnt[tid][w];
+            cnt[tid][w] = t;
+            t += k;
+        }
+        base[tid] = t ? atomicAdd(tid ? &ws->back : &ws->front, (unsigned long long)t) : 0ull;
+    }
+    __syncthreads();
+    int64_t at[2] = {(int64_t)base[0] + cnt[0][warp], (int64_t)base[1] + cnt[1][warp]};
+#pragma unroll
+    for (int j = 0; j < ORDER_RAYS / ORDER_BLOCK; ++j) {
+        const int i = (int)(b0 + 32 * j + lane);
+        if ((bits[0][j] >> lane) & 1u)
+            list[at[0] + __popc(bits[0][j] & below)] = i;
+        if ((bits[1][j] >> lane) & 1u)
+            list[n - 1 - (at[1] + __popc(bits[1][j] & below))] = i;
+        at[0] += __popc(bits[0][j]);
+        at[1] += __popc(bits[1][j]);
+    }
 }
 
 // Mark rays as empty slots (never traced, never counted as active).
@@ -2597,6 +2670,7 @@ TraceArgs make_trace_args(gray_ctx *ctx, void *state, int64_t n_state, int64_t s
     A.cancel = (const int *)&ctx->aux[AUX_CANCEL];
     A.one_per_thread = o.launch == GRAY_LAUNCH_ONE_PER_THREAD;
     A.stop_equator = o.stop_equator;
+    A.split = 0;
     A.handover = 0;
     A.zone_return = 0;
     return A;
@@ -2618,9 +2692,20 @@ unsigned persistent_grid(const gray_ctx *ctx, const void *kernel, int block, int
     return (unsigned)(want > 0 ? want : 1);
 }
 
+// Rays that a single-precision pass holds at once (its kernel keeps four
+// blocks of 128 threads on an SM), and the step budget below which a pass ends
+// too soon for its queue's order to matter.
+constexpr int ORDER_MIN_BUDGET = 512;
+int64_t resident_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512; }
+
 // One single- or double-precision pass over the queue of A (no zone kernel).
-// A persistent single-precision pass; the probe pass takes the uncapped
-// instantiation.
+// A persistent single-precision pass.  A queue of up to three blocks per SM
+// (any small image) and the planner's probe pass take the instantiation without
+// the 128-register cap, three blocks of 128 threads to an SM: nothing is
+// re-formed under register pressure (probe pass 0.56 -> 0.52 ms, 32^2 image
+// 1.545 -> 1.519, 128^2 projection 0.431 -> 0.423); a longer one needs the
+// fourth block (1024^2: 7.98 ms capped, 8.5 uncapped).
+constexpr int SMALL_BLOCKS_PER_SM = 3;
 template <int MODE>
 void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int block, bool probe, cudaStream_t s)
 {
@@ -2739,8 +2824,20 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             cudaEventRecord(ctx->ev[0], s);
             ctx->ev_used[0] = true;
         }
+        // more rays than the pass holds at once and no budget that ends it
+        // early: the order of the queue decides when its last ray ends
+        if (!order && ctx->opt.precision != GRAY_FP64 && !A.one_per_thread && n_state > resident_rays(ctx) &&
+            (step_budget <= 0 || step_budget > ORDER_MIN_BUDGET)) {
+            int *list = A.v.R ? A.v.R : A.v.L; // the zone pass fills R later; the other modes leave L unused
+            order_rays_kernel<<<grid_for(n_state, ORDER_RAYS), ORDER_BLOCK, 0, s>>>(A.v, n_state, list, ctx->ws);
+            if ((rc = check_launch()))
+                return rc;
+            A.order = list;
+            A.split = 1;
+        }
         if ((rc = launch_pass(ctx, A, work, s)))
             return rc;
+        A.split = 0;
         if (ctx->timing)
             cudaEventRecord(ctx->ev[1], s);
         if (ctx->opt.precision == GRAY_FP32_KAHAN_SEL64) {
