@@ -2709,7 +2709,7 @@ constexpr int SMALL_BLOCKS_PER_SM = 3;
 template <int MODE>
 void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int block, bool probe, cudaStream_t s)
 {
-    if (probe)
+    if (probe || work <= (int64_t)SMALL_BLOCKS_PER_SM * block * ctx->num_sms)
         trace32_kernel<MODE, 168>
             <<<persistent_grid(ctx, (const void *)trace32_kernel<MODE, 168>, block, work), block, 0, s>>>(A);
     else
