@@ -165,16 +165,16 @@ __device__ __forceinline__ void st_f4(void *p, int64_t i, float x, float y, floa
 
 // Workspace of one context (device memory, zeroed before each trace).
 struct Workspace {
-    unsigned long long head;    // next ray (or list slot) handed out by the queue of a pass
+    unsigned long long head[4]; // next ray (or list slot) handed out by the queue of each pass
     unsigned long long steps;   // steps taken in this call
     unsigned long long euler;   // Euler redos in this call
     unsigned long long fp64;    // steps taken in double by the selective mode in this call
     unsigned long long active;  // rays left active by this call
-    unsigned long long handoff; // rays appended to the hand-off list by the current pass
+    unsigned long long handoff[2]; // rays appended to the hand-off list by the first and the return pass
     unsigned long long demoted; // rays returned to single precision by the current zone pass
     unsigned long long zone_steps; // steps taken by the zone kernel in this call
     unsigned long long front, back; // lead-first queue: rays at its two ends
-    unsigned long long cancel;     // the cancel flag as the call ended (copied in by gray_trace)
+    unsigned long long cancel;     // the cancel flag as the call ended (copied in by count_active_kernel)
 };
 
 } // namespace
@@ -192,6 +192,7 @@ struct gray_ctx {
     cudaStream_t side = nullptr;       // gray_setup_plan: the planning passes (high priority)
     cudaEvent_t fork = nullptr, join = nullptr;
     cudaStream_t cancel_stream = nullptr; // gray_cancel writes the flag through it (non-blocking)
+    cudaMemPool_t pool = nullptr;      // small temporary tables; keeps its memory until gray_destroy
 };
 
 namespace {
@@ -212,6 +213,18 @@ struct ImageDev {
     float hc[8]; // single-precision per-ray constants (hole_constants_f), once per image
 };
 static_assert(sizeof(ImageDev) == 136, "gray_setup_noalloc's table size is documented in gray.h");
+
+// The image table of a call as a kernel argument: up to TABLE_INLINE images
+// travel in it, longer lists in device memory (`list`).  A single image then
+// needs no allocation and no copy; after a synchronisation the stream-ordered
+// allocator has given its memory back, and asking for it again took 105 us of
+// host time (32^2 image, 1.9 ms in all).
+constexpr int TABLE_INLINE = 8;
+struct ImageTable {
+    const ImageDev *list;
+    ImageDev one[TABLE_INLINE];
+    __device__ __forceinline__ const ImageDev *images() const { return list ? list : one; }
+};
 
 // Image-plane position of the ray in (row, col) of an image: a pixel centre
 // of the Cartesian grid, or the polar grid point of Sec. 4 (Eqs. 9-10).
@@ -277,9 +290,10 @@ __device__ void store_initial(const StateView &v, int prec, int64_t i, const dou
 // them: probe rays (every probe_stride-th pixel of each row and column,
 // which_probes = 1) or the others (which_probes = 0); probe_stride = 0 sets
 // up every ray.
-__global__ void setup_images_kernel(const ImageDev *imgs, int n_images, int64_t total, int64_t first_ray,
+__global__ void setup_images_kernel(const __grid_constant__ ImageTable T, int n_images, int64_t total, int64_t first_ray,
                                     StateView v, int prec, int probe_stride = 0, int which_probes = 0)
 {
+    const ImageDev *imgs = T.images();
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= total)
         return;
@@ -292,9 +306,10 @@ __global__ void setup_images_kernel(const ImageDev *imgs, int n_images, int64_t 
             hi = mid - 1;
     }
     const ImageDev im = imgs[lo];
-    const int64_t p = i - im.first;
-    const int64_t row = p / im.nx, col = p - row * im.nx;
-    if (probe_stride > 0 && ((row % probe_stride == 0 && col % probe_stride == 0) ? 1 : 0) != which_probes)
+    // a buffer holds fewer than 2^31 rays: 32-bit divisions
+    const unsigned p = (unsigned)(i - im.first), row = p / (unsigned)im.nx, col = p - row * (unsigned)im.nx;
+    if (probe_stride > 0 &&
+        ((row % (unsigned)probe_stride == 0 && col % (unsigned)probe_stride == 0) ? 1 : 0) != which_probes)
         return;
     double alpha, beta;
     image_point(im, row, col, alpha, beta);
@@ -569,6 +584,7 @@ struct TraceArgs {
     const int *order;                            // queue of ray indices, or NULL: 0 .. n-1
     int64_t n_queue;                             // queue length (order != NULL)
     const unsigned long long *n_queue_dev;       // if not NULL: queue length read on the device
+    unsigned long long *head, *handoff;          // the pass's counters in *ws: queue head, hand-off list length
     int64_t budget; // per-call step budget per ray, <= 0: none
     int max_steps;
     int refill;
@@ -703,7 +719,7 @@ template <int MODE, int MAXREG = 128> __global__ void __maxnreg__(MAXREG) trace3
             exhausted = true;
         if (SEL64) {
             int rank;
-            const unsigned long long hb = warp_count(&A.ws->handoff, pending, lane, &rank);
+            const unsigned long long hb = warp_count(A.handoff, pending, lane, &rank);
             if (pending)
                 v.L[hb + rank] = (int)id;
             pending = false;
@@ -718,7 +734,7 @@ template <int MODE, int MAXREG = 128> __global__ void __maxnreg__(MAXREG) trace3
             unsigned long long base = 0;
             if (!A.one_per_thread) {
                 if (lane == leader)
-                    base = atomicAdd(&A.ws->head, (unsigned long long)cnt);
+                    base = atomicAdd(A.head, (unsigned long long)cnt);
                 base = __shfl_sync(FULL, base, leader);
             }
             bool handoff_now = false;
@@ -772,7 +788,7 @@ template <int MODE, int MAXREG = 128> __global__ void __maxnreg__(MAXREG) trace3
             }
             if (SEL64) {
                 int rank;
-                const unsigned long long hb = warp_count(&A.ws->handoff, handoff_now, lane, &rank);
+                const unsigned long long hb = warp_count(A.handoff, handoff_now, lane, &rank);
                 if (handoff_now)
                     v.L[hb + rank] = (int)id;
             }
@@ -879,7 +895,7 @@ __global__ void __launch_bounds__(32) trace64_kernel(TraceArgs A)
             const int leader = __ffs(idle) - 1;
             unsigned long long base = 0;
             if (lane == leader)
-                base = atomicAdd(&A.ws->head, (unsigned long long)cnt);
+                base = atomicAdd(A.head, (unsigned long long)cnt);
             base = __shfl_sync(FULL, base, leader);
             if (!has) {
                 const int64_t slot = (int64_t)base + __popc(idle & ((1u << lane) - 1u));
@@ -914,7 +930,7 @@ __global__ void __launch_bounds__(32) trace64_kernel(TraceArgs A)
 
         if (give) {
             int rank;
-            const unsigned long long hb = warp_count(&A.ws->handoff, has, lane, &rank);
+            const unsigned long long hb = warp_count(A.handoff, has, lane, &rank);
             if (has) {
                 v.L[hb + rank] = (int)id;
                 st_d4(v.X, id, y[0], y[1], y[2], y[3]);
@@ -1001,7 +1017,7 @@ __global__ void __launch_bounds__(32) trace64_quad_kernel(TraceArgs A)
             const int leader = __ffs(idle) - 1;
             unsigned long long base = 0;
             if (lane == leader)
-                base = atomicAdd(&A.ws->head, (unsigned long long)cnt);
+                base = atomicAdd(A.head, (unsigned long long)cnt);
             base = __shfl_sync(FULL, base, leader);
             if (!has) {
                 const int64_t slot = (int64_t)base + __popc(idle & ((1u << (lane & 28)) - 1u));
@@ -1176,7 +1192,7 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
     Of.eps_xi = (float)A.eps_xi;
     Of.step_rule = A.step_rule;
     Of.stop_equator = A.stop_equator;
-    const int64_t n = (int64_t)*(volatile unsigned long long *)&A.ws->handoff;
+    const int64_t n = (int64_t)*(volatile unsigned long long *)A.handoff;
     const int epoch = *A.epoch_dev;
 
     bool has = false, exhausted = false, dbl = true;
@@ -1207,7 +1223,7 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
             const int leader = __ffs(idle) - 1;
             unsigned long long base = 0;
             if (lane == leader)
-                base = atomicAdd(&A.ws->head, (unsigned long long)cnt);
+                base = atomicAdd(A.head, (unsigned long long)cnt);
             base = __shfl_sync(FULL, base, leader);
             if (!has) {
                 const int64_t slot = (int64_t)base + __popc(idle & ((1u << lane) - 1u));
@@ -1470,17 +1486,35 @@ __global__ void range_stats_kernel(const int4 *S0, int64_t n, const long long *r
     }
 }
 
-// Rays still ACTIVE (for the per-call statistics).
-__global__ void count_active_kernel(const int4 *S0, int64_t n, unsigned long long *out)
+// Rays still ACTIVE (for the per-call statistics), and the cancel flag as the
+// passes ended, into the workspace.  One atomic per block: an atomic per warp
+// was most of its time (262144 rays: 7.7 -> 3 us).
+constexpr int COUNT_BLOCK = 256, COUNT_PER_THREAD = 4;
+__global__ void __launch_bounds__(COUNT_BLOCK) count_active_kernel(const int4 *S0, int64_t n, Workspace *ws,
+                                                                   const unsigned long long *cancel)
 {
-    unsigned long long mine = 0;
-    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
-        mine += (S0[i].x == GRAY_RAY_ACTIVE);
+    __shared__ int part[COUNT_BLOCK / 32];
+    int64_t mine = 0;
+    const int64_t stride = (int64_t)gridDim.x * COUNT_BLOCK;
+    for (int64_t i = (int64_t)blockIdx.x * COUNT_BLOCK + threadIdx.x; i < n; i += COUNT_PER_THREAD * stride) {
 #pragma unroll
-    for (int off = 16; off > 0; off >>= 1)
-        mine += __shfl_xor_sync(0xffffffffu, mine, off);
-    if ((threadIdx.x & 31) == 0 && mine)
-        atomicAdd(out, mine);
+        for (int j = 0; j < COUNT_PER_THREAD; ++j)
+            if (i + j * stride < n)
+                mine += S0[i + j * stride].x == GRAY_RAY_ACTIVE;
+    }
+    const int w = __reduce_add_sync(0xffffffffu, (int)mine);
+    if ((threadIdx.x & 31) == 0)
+        part[threadIdx.x >> 5] = w;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned long long t = 0;
+        for (int k = 0; k < COUNT_BLOCK / 32; ++k)
+            t += (unsigned long long)part[k];
+        if (t)
+            atomicAdd(&ws->active, t);
+        if (blockIdx.x == 0)
+            ws->cancel = *(volatile const unsigned long long *)cancel;
+    }
 }
 
 // --------------------------------------------------------------------------
@@ -1509,11 +1543,23 @@ constexpr int AUX_HIST = 1, AUX_OFF = 1 + PLAN_BUCKETS, AUX_WORDS = 1 + 2 * PLAN
 // one more word after the planning words: the call epoch (never cleared)
 constexpr int AUX_EPOCH = AUX_WORDS, AUX_CANCEL = AUX_WORDS + 1, AUX_ALLOC = AUX_WORDS + 2;
 
-// Start a new call: epochs run 1 .. 2^31 - 2 (0 marks a ray no call touched).
-__global__ void bump_epoch_kernel(unsigned long long *aux)
+// Start a new call in one launch: zero the workspace (every pass of the call
+// has counters of its own in it) and the first aux_words planning words, and
+// count the epoch up (epochs run 1 .. 2^31 - 2; 0 marks a ray no call touched).
+// A memset per pass and a kernel of one thread were five stream operations of
+// ~2 us each, on a frame of the view as long as its drawing.
+constexpr int BEGIN_BLOCK = 256;
+__global__ void __launch_bounds__(BEGIN_BLOCK) begin_call_kernel(Workspace *ws, unsigned long long *aux, int aux_words)
 {
-    int *e = (int *)&aux[AUX_EPOCH];
-    *e = (*e % 0x7ffffffe) + 1;
+    static_assert(sizeof(Workspace) % sizeof(unsigned long long) == 0, "the workspace is zeroed word by word");
+    for (int k = threadIdx.x; k < (int)(sizeof(Workspace) / sizeof(unsigned long long)); k += BEGIN_BLOCK)
+        ((unsigned long long *)ws)[k] = 0;
+    for (int k = threadIdx.x; k < aux_words; k += BEGIN_BLOCK)
+        aux[k] = 0;
+    if (threadIdx.x == 0) {
+        int *e = (int *)&aux[AUX_EPOCH];
+        *e = (*e % 0x7ffffffe) + 1;
+    }
 }
 
 __device__ __forceinline__ int image_of(const ImageDev *imgs, int n_images, int64_t i)
@@ -1533,9 +1579,10 @@ __device__ __forceinline__ int image_of(const ImageDev *imgs, int n_images, int6
 // row of each image), one thread per probe: its queue entry, and with `setup`
 // its initial state as setup_images_kernel writes it.  Probe q of the call
 // lies in the last image with probe_first <= q.
-__global__ void probe_rays_kernel(const ImageDev *imgs, int n_images, int64_t n_probes, int64_t first_ray,
+__global__ void probe_rays_kernel(const __grid_constant__ ImageTable T, int n_images, int64_t n_probes, int64_t first_ray,
                                   int stride, int *order, StateView v, int prec, int setup)
 {
+    const ImageDev *imgs = T.images();
     const int64_t q = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (q >= n_probes)
         return;
@@ -1548,9 +1595,9 @@ __global__ void probe_rays_kernel(const ImageDev *imgs, int n_images, int64_t n_
             hi = mid - 1;
     }
     const ImageDev im = imgs[lo];
-    const int64_t per_row = (im.nx + stride - 1) / stride;
-    const int64_t k = q - im.probe_first, row = (k / per_row) * stride, col = (k % per_row) * stride;
-    const int64_t i = im.first + row * im.nx + col;
+    const unsigned per_row = ((unsigned)im.nx + stride - 1) / stride;
+    const unsigned k = (unsigned)(q - im.probe_first), row = (k / per_row) * stride, col = (k % per_row) * stride;
+    const int64_t i = im.first + (int64_t)row * im.nx + col;
     order[q] = (int)(first_ray + i);
     if (setup) {
         double alpha, beta;
@@ -1570,8 +1617,8 @@ __device__ __forceinline__ int plan_bucket(const ImageDev *imgs, int n_images, i
                                            int stride, int budget, const int4 *S0)
 {
     const ImageDev im = imgs[image_of(imgs, n_images, i)];
-    const int64_t p = i - im.first, row = p / im.nx, col = p - row * im.nx;
-    const int64_t r0 = row - row % stride, c0 = col - col % stride;
+    const unsigned p = (unsigned)(i - im.first), row = p / (unsigned)im.nx, col = p - row * (unsigned)im.nx;
+    const int64_t r0 = row - row % (unsigned)stride, c0 = col - col % (unsigned)stride;
     float cost = 0.0f;
     for (int dr = -1; dr < 3; ++dr)
         for (int dc = -1; dc < 3; ++dc) {
@@ -1586,9 +1633,10 @@ __device__ __forceinline__ int plan_bucket(const ImageDev *imgs, int n_images, i
     return b < 0 ? 0 : (b >= PLAN_BUCKETS ? PLAN_BUCKETS - 1 : b);
 }
 
-__global__ void plan_hist_kernel(const ImageDev *imgs, int n_images, int64_t total, int64_t first_ray, int stride,
+__global__ void plan_hist_kernel(const __grid_constant__ ImageTable T, int n_images, int64_t total, int64_t first_ray, int stride,
                                  int budget, const int4 *S0, unsigned long long *aux)
 {
+    const ImageDev *imgs = T.images();
     __shared__ unsigned int h[PLAN_BUCKETS];
     for (int k = threadIdx.x; k < PLAN_BUCKETS; k += blockDim.x)
         h[k] = 0;
@@ -1622,9 +1670,10 @@ __global__ void __launch_bounds__(PLAN_BUCKETS) plan_scan_kernel(unsigned long l
 
 // Neighbouring pixels mostly share a bucket: the lanes of a warp with the
 // same bucket take their queue positions with one atomic (match + popc).
-__global__ void plan_scatter_kernel(const ImageDev *imgs, int n_images, int64_t total, int64_t first_ray, int stride,
+__global__ void plan_scatter_kernel(const __grid_constant__ ImageTable T, int n_images, int64_t total, int64_t first_ray, int stride,
                                     int budget, const int4 *S0, unsigned long long *aux, int *order)
 {
+    const ImageDev *imgs = T.images();
     const unsigned FULL = 0xffffffffu;
     const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     const bool valid = i < total;
@@ -1801,10 +1850,12 @@ __global__ void render_invariants_kernel(StateView v, int prec, int64_t first, i
 // on different addresses.
 constexpr int SHADOW_BLOCK = 256, SHADOW_RAYS = 2048, SHADOW_SEGMENTS = 4;
 
-__global__ void __launch_bounds__(SHADOW_BLOCK) shadow_accum_kernel(StateView v, int64_t first, const ImageDev *imgs,
+__global__ void __launch_bounds__(SHADOW_BLOCK) shadow_accum_kernel(StateView v, int64_t first,
+                                                                    const __grid_constant__ ImageTable T,
                                                                     int n_images, int64_t total,
                                                                     gray_shadow_info *out)
 {
+    const ImageDev *imgs = T.images();
     __shared__ unsigned long long part[5][SHADOW_BLOCK / 32];
     const int64_t b0 = (int64_t)blockIdx.x * SHADOW_RAYS;
     const int64_t b1 = total - b0 < SHADOW_RAYS ? total : b0 + SHADOW_RAYS;
@@ -1872,8 +1923,9 @@ __global__ void __launch_bounds__(SHADOW_BLOCK) shadow_accum_kernel(StateView v,
     }
 }
 
-__global__ void shadow_final_kernel(const ImageDev *imgs, int n_images, gray_shadow_info *out)
+__global__ void shadow_final_kernel(const __grid_constant__ ImageTable T, int n_images, gray_shadow_info *out)
 {
+    const ImageDev *imgs = T.images();
     int k = blockIdx.x * blockDim.x + threadIdx.x;
     if (k >= n_images)
         return;
@@ -2099,11 +2151,25 @@ struct CamDev {
     int width, height, ortho, mask;
 };
 
-__global__ void fill_kernel(unsigned *p, int64_t n, unsigned value)
+// Zero the counts and set the depths to +inf (depth may be NULL) in one pass
+// of 16-byte stores; images off a 16-byte boundary word by word.
+__global__ void clear_images_kernel(unsigned *count, float *depth, int64_t n)
 {
-    const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    if (i < n)
-        p[i] = value;
+    const int64_t i = 4 * ((int64_t)blockIdx.x * blockDim.x + threadIdx.x);
+    if (i >= n)
+        return;
+    const float inf = __int_as_float(0x7f800000);
+    if (i + 4 <= n && (((uintptr_t)count | (uintptr_t)depth) & 15) == 0) {
+        *(uint4 *)(count + i) = make_uint4(0u, 0u, 0u, 0u);
+        if (depth)
+            *(float4 *)(depth + i) = make_float4(inf, inf, inf, inf);
+        return;
+    }
+    for (int64_t j = i; j < i + 4 && j < n; ++j) {
+        count[j] = 0u;
+        if (depth)
+            depth[j] = inf;
+    }
 }
 
 // Deposit one sprite at image position (x, y) with depth z.
@@ -2477,16 +2543,59 @@ std::vector<ImageDev> image_table(const gray_image *images, int n_images, int64_
     return t;
 }
 
-// Copy a small host table to the device on `stream` through a temporary
-// buffer that is freed after the stream reaches it.
-int upload_table(const void *host, size_t bytes, cudaStream_t s, void **dev)
+// A temporary buffer on `stream` from the context's own pool, which keeps its
+// memory between calls (the device's default pool gives it back at every
+// synchronisation).  Freed with cudaFreeAsync.  Under stream capture the
+// default pool serves, as a pool cannot be created there.
+int pool_alloc(gray_ctx *ctx, void **dev, size_t bytes, cudaStream_t s)
 {
     *dev = nullptr;
-    if (cudaMallocAsync(dev, bytes, s) != cudaSuccess)
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(s, &capture) != cudaSuccess)
         return GRAY_ECUDA;
-    if (cudaMemcpyAsync(*dev, host, bytes, cudaMemcpyHostToDevice, s) != cudaSuccess)
-        return GRAY_ECUDA;
-    return GRAY_OK;
+    if (capture != cudaStreamCaptureStatusNone)
+        return cuda_err(cudaMallocAsync(dev, bytes, s));
+    if (!ctx->pool) {
+        cudaMemPoolProps props = {};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = ctx->device;
+        uint64_t keep = UINT64_MAX;
+        if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess)
+            return GRAY_ECUDA;
+        if (cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
+            return GRAY_ECUDA;
+    }
+    return cuda_err(cudaMallocFromPoolAsync(dev, bytes, ctx->pool, s));
+}
+
+// Copy a small host table to the device on `stream` through a temporary
+// buffer that is freed after the stream reaches it.
+int upload_table(gray_ctx *ctx, const void *host, size_t bytes, cudaStream_t s, void **dev)
+{
+    const int rc = pool_alloc(ctx, dev, bytes, s);
+    if (rc)
+        return rc;
+    return cuda_err(cudaMemcpyAsync(*dev, host, bytes, cudaMemcpyHostToDevice, s));
+}
+
+// The image table of a call as a kernel argument (see ImageTable); released
+// after the kernels that take it.
+int stage_images(gray_ctx *ctx, const std::vector<ImageDev> &t, cudaStream_t s, ImageTable &T)
+{
+    T.list = nullptr;
+    if (t.size() <= (size_t)TABLE_INLINE) {
+        std::copy(t.begin(), t.end(), T.one);
+        return GRAY_OK;
+    }
+    void *dev = nullptr;
+    const int rc = upload_table(ctx, t.data(), t.size() * sizeof(ImageDev), s, &dev);
+    T.list = (const ImageDev *)dev;
+    return rc;
+}
+int release_images(const ImageTable &T, cudaStream_t s)
+{
+    return T.list ? cuda_err(cudaFreeAsync((void *)T.list, s)) : GRAY_OK;
 }
 
 } // namespace
@@ -2591,6 +2700,8 @@ void gray_destroy(gray_ctx *ctx)
     cudaFree(ctx->aux);
     if (ctx->cancel_stream)
         cudaStreamDestroy(ctx->cancel_stream);
+    if (ctx->pool)
+        cudaMemPoolDestroy(ctx->pool); // its memory goes once the frees queued on the streams are done
     cudaFreeHost(ctx->ws_host);
     delete ctx;
 }
@@ -2611,17 +2722,14 @@ int gray_setup(gray_ctx *ctx, const gray_image *images, int32_t n_images, void *
     if (first_ray + total > n_state)
         return GRAY_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    void *dimg = nullptr;
-    if ((rc = upload_table(t.data(), t.size() * sizeof(ImageDev), s, &dimg)))
+    ImageTable T;
+    if ((rc = stage_images(ctx, t, s, T)))
         return rc;
     StateView v = make_view(state, n_state, ctx->opt.precision);
-    setup_images_kernel<<<grid_for(total, 256), 256, 0, s>>>((const ImageDev *)dimg, n_images, total, first_ray, v,
-                                                           ctx->opt.precision);
+    setup_images_kernel<<<grid_for(total, 256), 256, 0, s>>>(T, n_images, total, first_ray, v, ctx->opt.precision);
     rc = check_launch();
-    cudaError_t e = cudaFreeAsync(dimg, s);
-    if (rc)
-        return rc;
-    return cuda_err(e);
+    const int rf = release_images(T, s);
+    return rc ? rc : rf;
 }
 
 int gray_setup_rays(gray_ctx *ctx, const double *rays, int64_t n, double M, void *state, size_t state_bytes,
@@ -2667,6 +2775,8 @@ TraceArgs make_trace_args(gray_ctx *ctx, void *state, int64_t n_state, int64_t s
     A.r_esc_frac = o.r_esc_frac;
     A.r_sw = o.r_sw;
     A.ws = ctx->ws;
+    A.head = &ctx->ws->head[0];
+    A.handoff = &ctx->ws->handoff[0];
     A.cancel = (const int *)&ctx->aux[AUX_CANCEL];
     A.one_per_thread = o.launch == GRAY_LAUNCH_ONE_PER_THREAD;
     A.stop_equator = o.stop_equator;
@@ -2746,10 +2856,9 @@ int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
             return rc;
         A.handover = 0;
         A.order = A.v.L;
-        A.n_queue_dev = &ctx->ws->handoff;
+        A.n_queue_dev = A.handoff;
+        A.head = &ctx->ws->head[1];
         quad_work = QUAD_HANDOVER_PER_SM * sms; // at most; the kernel reads the list's length
-        if (cudaMemsetAsync(&ctx->ws->head, 0, sizeof(unsigned long long), s) != cudaSuccess)
-            return GRAY_ECUDA;
     }
     per_sm = ctx->opt.blocks_per_sm > 0 ? per_sm : QUAD_PER_SM;
     trace64_quad_kernel<<<(unsigned)std::min(per_sm * sms, (quad_work + 7) / 8), 32, 0, s>>>(A);
@@ -2807,9 +2916,7 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
     if (order ? n_order < 0 : n_order != 0)
         return GRAY_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    if (cudaMemsetAsync(ctx->ws, 0, sizeof(Workspace), s) != cudaSuccess)
-        return GRAY_ECUDA;
-    bump_epoch_kernel<<<1, 1, 0, s>>>(ctx->aux);
+    begin_call_kernel<<<1, BEGIN_BLOCK, 0, s>>>(ctx->ws, ctx->aux, 0);
     if ((rc = check_launch()))
         return rc;
     TraceArgs A = make_trace_args(ctx, state, n_state, step_budget);
@@ -2851,15 +2958,16 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             TraceArgs Z = A;
             Z.refill = 1;
             Z.zone_return = 1;
+            Z.head = &ctx->ws->head[1];
             TraceArgs B = A;
             B.order = A.v.R;
             B.n_queue_dev = &ctx->ws->demoted;
+            B.head = &ctx->ws->head[2];
+            B.handoff = &ctx->ws->handoff[1];
             if (ctx->timing) {
                 cudaEventRecord(ctx->ev[2], s);
                 ctx->ev_used[1] = true;
             }
-            if (cudaMemsetAsync(&ctx->ws->head, 0, sizeof(unsigned long long), s) != cudaSuccess)
-                return GRAY_ECUDA;
             // one block per SM: the double pipe is shared by the SM and a warp
             // instruction holds it whatever its active lanes, so few warps,
             // each draining many zone rays, waste the fewest pipe cycles on
@@ -2872,14 +2980,11 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             if ((rc = check_launch()))
                 return rc;
             // the hand-off list is consumed: pass B appends to it from 0
-            if (cudaMemsetAsync(&ctx->ws->head, 0, sizeof(unsigned long long), s) != cudaSuccess ||
-                cudaMemsetAsync(&ctx->ws->handoff, 0, sizeof(unsigned long long), s) != cudaSuccess)
-                return GRAY_ECUDA;
             if ((rc = launch_pass(ctx, B, work, s)))
                 return rc;
-            if (cudaMemsetAsync(&ctx->ws->head, 0, sizeof(unsigned long long), s) != cudaSuccess)
-                return GRAY_ECUDA;
             Z.zone_return = 0;
+            Z.head = &ctx->ws->head[3];
+            Z.handoff = &ctx->ws->handoff[1];
             if (ctx->opt.zone_arith == GRAY_ZONE_FP64)
                 zone_kernel<false, double>
                     <<<persistent_grid(ctx, (const void *)zone_kernel<false, double>, block, work), block, 0, s>>>(Z);
@@ -2894,16 +2999,14 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
     }
     if (!n_active_host && !stats_host)
         return 1;
-    if (n_state > 0) {
-        count_active_kernel<<<grid_for(n_state, 256) < 1024 ? grid_for(n_state, 256) : 1024, 256, 0, s>>>(
-            A.v.S0, n_state, &ctx->ws->active);
+    {
+        const int64_t blocks = (n_state + COUNT_BLOCK * COUNT_PER_THREAD - 1) / (COUNT_BLOCK * COUNT_PER_THREAD);
+        count_active_kernel<<<(unsigned)std::min<int64_t>(std::max<int64_t>(blocks, 1), 8 * ctx->num_sms), COUNT_BLOCK, 0,
+                              s>>>(A.v.S0, n_state, ctx->ws, &ctx->aux[AUX_CANCEL]);
         if ((rc = check_launch()))
             return rc;
     }
-    // the cancel flag as the passes ended, into the workspace's last word
-    if (cudaMemcpyAsync(&ctx->ws->cancel, &ctx->aux[AUX_CANCEL], sizeof(unsigned long long),
-                        cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
-        cudaMemcpyAsync(ctx->ws_host, ctx->ws, sizeof(Workspace), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+    if (cudaMemcpyAsync(ctx->ws_host, ctx->ws, sizeof(Workspace), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
         cudaStreamSynchronize(s) != cudaSuccess)
         return GRAY_ECUDA;
     const Workspace &w = *ctx->ws_host;
@@ -2952,25 +3055,22 @@ int plan_args(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, c
     return GRAY_OK;
 }
 
-// The planning passes on stream s (image table `im` already on the device):
+// The planning passes on stream s (image table T):
 // 1. the probe list (written into the order buffer; with setup_probes the
 // probe rays are set up in the same pass), 2. the probes traced under the
 // probe budget, 3. predicted cost -> bucket histogram -> descending offsets
 // -> queue.  Only the probe rays' states are read.
-int plan_passes(gray_ctx *ctx, void *state, int64_t n_state, int32_t n_images, const ImageDev *im, int64_t total,
+int plan_passes(gray_ctx *ctx, void *state, int64_t n_state, int32_t n_images, const ImageTable &T, int64_t total,
                 int64_t n_probes, int64_t first_ray, int32_t probe_stride, int32_t probe_budget, int32_t *order,
                 bool setup_probes, cudaStream_t s)
 {
     int rc;
-    if (cudaMemsetAsync(ctx->aux, 0, AUX_WORDS * sizeof(unsigned long long), s) != cudaSuccess ||
-        cudaMemsetAsync(ctx->ws, 0, sizeof(Workspace), s) != cudaSuccess)
-        return GRAY_ECUDA;
-    const StateView v = make_view(state, n_state, ctx->opt.precision);
-    probe_rays_kernel<<<grid_for(n_probes, 128), 128, 0, s>>>(im, n_images, n_probes, first_ray, probe_stride, order,
-                                                             v, ctx->opt.precision, setup_probes ? 1 : 0);
+    begin_call_kernel<<<1, BEGIN_BLOCK, 0, s>>>(ctx->ws, ctx->aux, AUX_WORDS);
     if ((rc = check_launch()))
         return rc;
-    bump_epoch_kernel<<<1, 1, 0, s>>>(ctx->aux);
+    const StateView v = make_view(state, n_state, ctx->opt.precision);
+    probe_rays_kernel<<<grid_for(n_probes, 128), 128, 0, s>>>(T, n_images, n_probes, first_ray, probe_stride, order,
+                                                             v, ctx->opt.precision, setup_probes ? 1 : 0);
     if ((rc = check_launch()))
         return rc;
     TraceArgs A = make_trace_args(ctx, state, n_state, probe_budget);
@@ -2985,14 +3085,14 @@ int plan_passes(gray_ctx *ctx, void *state, int64_t n_state, int32_t n_images, c
         return rc;
     if (ctx->timing)
         cudaEventRecord(ctx->ev[5], s);
-    plan_hist_kernel<<<grid_for(total, 256), 256, 0, s>>>(im, n_images, total, first_ray, probe_stride, probe_budget,
+    plan_hist_kernel<<<grid_for(total, 256), 256, 0, s>>>(T, n_images, total, first_ray, probe_stride, probe_budget,
                                                          v.S0, ctx->aux);
     if ((rc = check_launch()))
         return rc;
     plan_scan_kernel<<<1, PLAN_BUCKETS, 0, s>>>(ctx->aux);
     if ((rc = check_launch()))
         return rc;
-    plan_scatter_kernel<<<grid_for(total, 256), 256, 0, s>>>(im, n_images, total, first_ray, probe_stride,
+    plan_scatter_kernel<<<grid_for(total, 256), 256, 0, s>>>(T, n_images, total, first_ray, probe_stride,
                                                             probe_budget, v.S0, ctx->aux, order);
     return check_launch();
 }
@@ -3012,15 +3112,13 @@ int gray_plan(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, c
     if (rc)
         return rc;
     cudaStream_t s = (cudaStream_t)stream;
-    void *dimg = nullptr;
-    if ((rc = upload_table(t.data(), t.size() * sizeof(ImageDev), s, &dimg)))
+    ImageTable T;
+    if ((rc = stage_images(ctx, t, s, T)))
         return rc;
-    rc = plan_passes(ctx, state, n_state, n_images, (const ImageDev *)dimg, total, n_probes, first_ray, probe_stride,
-                     probe_budget, order, false, s);
-    cudaError_t e = cudaFreeAsync(dimg, s);
-    if (rc)
-        return rc;
-    return cuda_err(e);
+    rc = plan_passes(ctx, state, n_state, n_images, T, total, n_probes, first_ray, probe_stride, probe_budget, order,
+                     false, s);
+    const int rf = release_images(T, s);
+    return rc ? rc : rf;
 }
 
 int gray_setup_plan(gray_ctx *ctx, const gray_image *images, int32_t n_images, void *state, size_t state_bytes,
@@ -3041,10 +3139,9 @@ int gray_setup_plan(gray_ctx *ctx, const gray_image *images, int32_t n_images, v
         (!ctx->join && cudaEventCreateWithFlags(&ctx->join, cudaEventDisableTiming) != cudaSuccess))
         return GRAY_ECUDA;
     cudaStream_t s = (cudaStream_t)stream;
-    void *dimg = nullptr;
-    if ((rc = upload_table(t.data(), t.size() * sizeof(ImageDev), s, &dimg)))
+    ImageTable T;
+    if ((rc = stage_images(ctx, t, s, T)))
         return rc;
-    const ImageDev *im = (const ImageDev *)dimg;
     StateView v = make_view(state, n_state, ctx->opt.precision);
     // the probe rays' set-up and the planning passes on the context's
     // high-priority stream, after everything queued so far on the caller's
@@ -3055,11 +3152,11 @@ int gray_setup_plan(gray_ctx *ctx, const gray_image *images, int32_t n_images, v
         if (cudaEventRecord(ctx->fork, s) != cudaSuccess || cudaStreamWaitEvent(ctx->side, ctx->fork, 0) != cudaSuccess) {
             rc = GRAY_ECUDA;
         } else {
-            rc = plan_passes(ctx, state, n_state, n_images, im, total, n_probes, first_ray, probe_stride, probe_budget,
+            rc = plan_passes(ctx, state, n_state, n_images, T, total, n_probes, first_ray, probe_stride, probe_budget,
                              order, true, ctx->side);
             const bool joined = cudaEventRecord(ctx->join, ctx->side) == cudaSuccess;
             if (!rc) {
-                setup_images_kernel<<<grid_for(total, 256), 256, 0, s>>>(im, n_images, total, first_ray, v,
+                setup_images_kernel<<<grid_for(total, 256), 256, 0, s>>>(T, n_images, total, first_ray, v,
                                                                        ctx->opt.precision, probe_stride, 0);
                 rc = check_launch();
             }
@@ -3073,10 +3170,8 @@ int gray_setup_plan(gray_ctx *ctx, const gray_image *images, int32_t n_images, v
             }
         }
     }
-    cudaError_t e = cudaFreeAsync(dimg, s);
-    if (rc)
-        return rc;
-    return cuda_err(e);
+    const int rf = release_images(T, s);
+    return rc ? rc : rf;
 }
 
 int gray_cancel(gray_ctx *ctx, int32_t on)
@@ -3156,9 +3251,9 @@ int gray_count_active(gray_ctx *ctx, const void *state, size_t state_bytes, int6
         return GRAY_OK;
     cudaStream_t s = (cudaStream_t)stream;
     void *dr = nullptr, *dc = nullptr;
-    if ((rc = upload_table(ranges, 2 * sizeof(int64_t) * (size_t)n_ranges, s, &dr)))
+    if ((rc = upload_table(ctx, ranges, 2 * sizeof(int64_t) * (size_t)n_ranges, s, &dr)))
         return rc;
-    if (cudaMallocAsync(&dc, 2 * sizeof(unsigned long long) * (size_t)n_ranges, s) != cudaSuccess) {
+    if (pool_alloc(ctx, &dc, 2 * sizeof(unsigned long long) * (size_t)n_ranges, s) != GRAY_OK) {
         cudaFreeAsync(dr, s);
         return GRAY_ECUDA;
     }
@@ -3240,22 +3335,20 @@ int gray_shadow(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_
     if (first_ray + total > n_state)
         return GRAY_EINVAL;
     cudaStream_t s = (cudaStream_t)stream;
-    void *dimg = nullptr;
-    if ((rc = upload_table(t.data(), t.size() * sizeof(ImageDev), s, &dimg)))
+    ImageTable T;
+    if ((rc = stage_images(ctx, t, s, T)))
         return rc;
     if (cudaMemsetAsync(out, 0, sizeof(gray_shadow_info) * (size_t)n_images, s) != cudaSuccess)
         return GRAY_ECUDA;
     StateView v = make_view((void *)state, n_state, ctx->opt.precision);
-    shadow_accum_kernel<<<grid_for(total, SHADOW_RAYS), SHADOW_BLOCK, 0, s>>>(v, first_ray, (const ImageDev *)dimg,
-                                                                             n_images, total, out);
+    shadow_accum_kernel<<<grid_for(total, SHADOW_RAYS), SHADOW_BLOCK, 0, s>>>(v, first_ray, T, n_images, total,
+                                                                             out);
     if ((rc = check_launch()))
         return rc;
-    shadow_final_kernel<<<grid_for(n_images, 128), 128, 0, s>>>((const ImageDev *)dimg, n_images, out);
+    shadow_final_kernel<<<grid_for(n_images, 128), 128, 0, s>>>(T, n_images, out);
     rc = check_launch();
-    cudaError_t e = cudaFreeAsync(dimg, s);
-    if (rc)
-        return rc;
-    return cuda_err(e);
+    const int rf = release_images(T, s);
+    return rc ? rc : rf;
 }
 
 int gray_ring(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_state, int64_t first_ray,
@@ -3296,7 +3389,7 @@ int gray_ring(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_st
     const size_t table_bytes = (sizeof(RingDev) * t.size() + 255) & ~(size_t)255;
     const size_t scratch = table_bytes + (boundary ? 0 : sizeof(double) * (size_t)rows);
     void *dmem = nullptr;
-    if (cudaMallocAsync(&dmem, scratch, s) != cudaSuccess)
+    if (pool_alloc(ctx, &dmem, scratch, s) != GRAY_OK)
         return GRAY_ECUDA;
     const RingDev *dimg = (const RingDev *)dmem;
     double *rb = boundary ? boundary : (double *)((char *)dmem + table_bytes);
@@ -3373,13 +3466,9 @@ int gray_splat(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_s
     c.mask = cam->status_mask;
     cudaStream_t st = (cudaStream_t)stream;
     if (cam->clear) {
-        if (cudaMemsetAsync(count, 0, sizeof(uint32_t) * (size_t)npix, st) != cudaSuccess)
-            return GRAY_ECUDA;
-        if (depth) {
-            fill_kernel<<<grid_for(npix, 256), 256, 0, st>>>((unsigned *)depth, npix, 0x7f800000u);
-            if ((rc = check_launch()))
-                return rc;
-        }
+        clear_images_kernel<<<grid_for((npix + 3) / 4, 256), 256, 0, st>>>(count, depth, npix);
+        if ((rc = check_launch()))
+            return rc;
     }
     if (n == 0)
         return GRAY_OK;
@@ -3489,8 +3578,9 @@ int gray_setup_noalloc(int32_t precision, const gray_image *images, int32_t n_im
             return GRAY_ECUDA;
     }
     StateView v = make_view(state, n_state, precision);
-    setup_images_kernel<<<grid_for(total, 256), 256, 0, s>>>((const ImageDev *)table, n_images, total, first_ray, v,
-                                                           precision);
+    ImageTable T;
+    T.list = (const ImageDev *)table;
+    setup_images_kernel<<<grid_for(total, 256), 256, 0, s>>>(T, n_images, total, first_ray, v, precision);
     return check_launch();
 }
 
