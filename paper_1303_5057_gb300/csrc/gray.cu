@@ -2815,15 +2815,28 @@ int64_t resident_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512;
 // re-formed under register pressure (probe pass 0.56 -> 0.52 ms, 32^2 image
 // 1.545 -> 1.519, 128^2 projection 0.431 -> 0.423); a longer one needs the
 // fourth block (1024^2: 7.98 ms capped, 8.5 uncapped).
-constexpr int SMALL_BLOCKS_PER_SM = 3;
+//
+// A probe pass beside the set-up of the other rays (gray_setup_plan) must
+// leave it room: three uncapped blocks take the whole register file, and the
+// set-up, bound by the FP64 pipe that the probes leave idle, then waited for
+// them.  A long probe queue takes two capped blocks per SM there (24 images,
+// 2.4 M rays: set-up and plan 1.84 -> 1.39 ms; 64 images, 25 M rays: 17.5 ->
+// 12.1, of which the set-up alone is 10.5; three capped blocks 1.52 and 14.1,
+// two uncapped ones 1.57 and 13.7).
+enum class Pass { Main, Probe, ProbeBesideSetup };
+constexpr int SMALL_BLOCKS_PER_SM = 3, BESIDE_BLOCKS_PER_SM = 2;
 template <int MODE>
-void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int block, bool probe, cudaStream_t s)
+void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int block, Pass pass, cudaStream_t s)
 {
-    if (probe || work <= (int64_t)SMALL_BLOCKS_PER_SM * block * ctx->num_sms)
+    const int64_t sms = ctx->num_sms;
+    const bool beside = pass == Pass::ProbeBesideSetup && work > BESIDE_BLOCKS_PER_SM * block * sms;
+    if (!beside && (pass != Pass::Main || work <= SMALL_BLOCKS_PER_SM * block * sms)) {
         trace32_kernel<MODE, 168>
             <<<persistent_grid(ctx, (const void *)trace32_kernel<MODE, 168>, block, work), block, 0, s>>>(A);
-    else
-        trace32_kernel<MODE><<<persistent_grid(ctx, (const void *)trace32_kernel<MODE>, block, work), block, 0, s>>>(A);
+        return;
+    }
+    const unsigned grid = persistent_grid(ctx, (const void *)trace32_kernel<MODE>, block, work);
+    trace32_kernel<MODE><<<beside ? std::min(grid, (unsigned)(BESIDE_BLOCKS_PER_SM * sms)) : grid, block, 0, s>>>(A);
 }
 
 // A double-precision pass.  An SM takes one FP64 instruction per 19 cycles and
@@ -2865,8 +2878,7 @@ int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
     return check_launch();
 }
 
-// probe: the planner's probe pass (the uncapped instantiation).
-int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s, bool probe = false)
+int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s, Pass pass = Pass::Main)
 {
     if (A.one_per_thread && ctx->opt.precision != GRAY_FP64) {
         // the paper's launch (Eq. 1): n_grid = floor((n - 1) / n_block) + 1
@@ -2891,13 +2903,13 @@ int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s,
     case GRAY_FP64:
         return launch_trace64(ctx, A, work, s);
     case GRAY_FP32:
-        launch_trace32<GRAY_FP32>(ctx, A, work, block, probe, s);
+        launch_trace32<GRAY_FP32>(ctx, A, work, block, pass, s);
         break;
     case GRAY_FP32_KAHAN:
-        launch_trace32<GRAY_FP32_KAHAN>(ctx, A, work, block, probe, s);
+        launch_trace32<GRAY_FP32_KAHAN>(ctx, A, work, block, pass, s);
         break;
     default:
-        launch_trace32<GRAY_FP32_KAHAN_SEL64>(ctx, A, work, block, probe, s);
+        launch_trace32<GRAY_FP32_KAHAN_SEL64>(ctx, A, work, block, pass, s);
         break;
     }
     return check_launch();
@@ -3081,7 +3093,7 @@ int plan_passes(gray_ctx *ctx, void *state, int64_t n_state, int32_t n_images, c
         cudaEventRecord(ctx->ev[4], s);
         ctx->ev_used[2] = true;
     }
-    if ((rc = launch_pass(ctx, A, n_probes, s, true)))
+    if ((rc = launch_pass(ctx, A, n_probes, s, setup_probes ? Pass::ProbeBesideSetup : Pass::Probe)))
         return rc;
     if (ctx->timing)
         cudaEventRecord(ctx->ev[5], s);
