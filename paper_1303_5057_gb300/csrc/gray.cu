@@ -1182,7 +1182,7 @@ template <typename T> __device__ __forceinline__ void load_zone_state(const Stat
 // The switches are exact one way (hi - lo to T) and a rounding the other way
 // (T to hi, lo; exact for double-single), the same in both forms, so a ray's
 // arithmetic does not depend on which pass runs it.
-template <bool RETURN, typename T>
+template <bool RETURN, typename T, int CFG = CFG_EQUATOR>
 __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
 {
     using Z = ZoneArith<T>;
@@ -1193,8 +1193,8 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
     Od.h_frac = T(A.h_frac);
     Od.h_min = T(A.h_min);
     Od.eps_xi = T(A.eps_xi);
-    Od.step_rule = A.step_rule;
-    Od.stop_equator = A.stop_equator;
+    Od.step_rule = CFG == CFG_EQUATOR ? A.step_rule : CFG == CFG_EQ2 ? GRAY_STEP_EQ2 : GRAY_STEP_BENCH;
+    Od.stop_equator = CFG == CFG_EQUATOR ? A.stop_equator : 0;
     StepOpt<float> Of;
     Of.h_frac = (float)A.h_frac;
     Of.h_min = (float)A.h_min;
@@ -3028,7 +3028,12 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             if (ctx->opt.zone_arith == GRAY_ZONE_FP64)
                 zone_kernel<true, double><<<(unsigned)ctx->num_sms, block, 0, s>>>(Z);
             else
-                zone_kernel<true, ds><<<(unsigned)ctx->num_sms, block, 0, s>>>(Z);
+            {
+                const auto kernel = Z.stop_equator ? zone_kernel<true, ds, CFG_EQUATOR>
+                                    : Z.step_rule == GRAY_STEP_EQ2 ? zone_kernel<true, ds, CFG_EQ2>
+                                                                   : zone_kernel<true, ds, CFG_BENCH>;
+                kernel<<<(unsigned)ctx->num_sms, block, 0, s>>>(Z);
+            }
             if ((rc = check_launch()))
                 return rc;
             // the hand-off list is consumed: pass B appends to it from 0

@@ -728,6 +728,32 @@ __device__ __forceinline__ bool xi_fails_ds(const float *y1, const float *c1, fl
     return !(fabsf(norm.hi + norm.lo) <= eps * fabsf(gtt * (kt * kt)));
 }
 
+// The Eq. 4 test of a double-single state.  Its high words decide it in single
+// precision (25 instructions) unless |g(k, k)| lies within 2^-17 of its terms'
+// size of the threshold -- eight times the flag of the single-precision
+// tracer's own test, as v = (r^2 + a^2) k^ph - a k^t cancels more this close to
+// the horizon; then the double-single form (190 instructions) does.
+__device__ __forceinline__ bool xi_fails(const Hole<ds> &H, const Geo<ds> &g, const ds *y, ds eps)
+{
+    Hole<float> h;
+    h.a = H.a.hi;
+    h.a2 = H.a2.hi;
+    h.m2M = H.m2M.hi;
+    Geo<float> f;
+    f.r = g.r.hi;
+    f.s = g.s.hi;
+    f.Sigma = g.Sigma.hi;
+    f.Delta = g.Delta.hi;
+    f.iS = g.iS.hi;
+    f.iD = g.iD.hi;
+    const float k[8] = {0.0f, 0.0f, 0.0f, 0.0f, y[4].hi, y[5].hi, y[6].hi, y[7].hi};
+    const NormF n = null_norm_f(h, f, k);
+    const float thr = eps.hi * fabsf(n.den);
+    if (fabsf(fabsf(n.norm) - thr) > 7.62939453125e-6f * n.size) // false for NaN
+        return fabsf(n.norm) > thr;
+    return xi_fails<ds>(H, g, y, eps);
+}
+
 // dk^mu/dl = -Gamma^mu_ab k^a k^b, from the closed-form symbols grouped with
 // w = k^t - a s^2 k^ph.  Inputs: r, theta and k = (kt, kr, kh, kp).
 template <typename T>
