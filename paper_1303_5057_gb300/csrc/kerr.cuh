@@ -622,6 +622,7 @@ __device__ __forceinline__ ds operator*(ds a, ds b) { return ds_mul(a, b); }
 __device__ __forceinline__ ds operator/(ds a, ds b) { return ds_mul(a, ds_recip(b)); }
 __device__ __forceinline__ bool operator<(ds a, ds b) { return a.hi < b.hi || (a.hi == b.hi && a.lo < b.lo); }
 __device__ __forceinline__ bool operator>(ds a, ds b) { return b < a; }
+__device__ __forceinline__ bool operator==(ds a, ds b) { return a.hi == b.hi && a.lo == b.lo; }
 __device__ __forceinline__ bool operator<=(ds a, ds b) { return !(b < a) && a.hi == a.hi && b.hi == b.hi; }
 __device__ __forceinline__ bool operator>=(ds a, ds b) { return b <= a; }
 __device__ __forceinline__ ds fma(ds a, ds b, ds c) { return ds_fma(a, b, c); }
@@ -799,7 +800,9 @@ template <typename T> __device__ __forceinline__ T hermite(T x0, T v0, T x1, T v
 // small over one step, onto the root the oracle's bisection finds (8 and 16
 // iterations pass the same parity tests; each costs the zone pass ~1.5 %).
 // Single:
-// Newton's method, 6 iterations.
+// Newton's method, 6 iterations.  Both stop early once s repeats: the rest
+// would repeat it (the bracket only closes on s itself), so the bits are those
+// of the full count (usually reached after 2 - 3 Newton steps).
 template <typename T>
 __device__ __forceinline__ T crossing_fraction(const T *y0, const T *y1, T h, T target, int m = 1)
 {
@@ -824,6 +827,8 @@ __device__ __forceinline__ T crossing_fraction(const T *y0, const T *y1, T h, T 
             T sn = s - f * idf;
             if (!(sn >= lo && sn <= hi))
                 sn = T(0.5) * (lo + hi);
+            if (sn == s)
+                break;
             s = sn;
         }
         return s;
@@ -845,6 +850,8 @@ __device__ __forceinline__ T crossing_fraction(const T *y0, const T *y1, T h, T 
         T sn = s - f / df;
         if (!(sn >= lo && sn <= hi)) // inclusive: f = 0 keeps s (the root)
             sn = T(0.5) * (lo + hi);
+        if (sn == s)
+            break;
         s = sn;
     }
     return s;
