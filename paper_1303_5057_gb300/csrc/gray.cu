@@ -163,6 +163,48 @@ __device__ __forceinline__ void st_f4(void *p, int64_t i, float x, float y, floa
     ((float4 *)p)[i] = make_float4(x, y, z, w);
 }
 
+// Conversions between double and single precision or integers on the integer
+// and FP32 pipes, exact as the instructions are: those run on the FP64 pipe of
+// this part, 19 cycles of an SM per warp, which the set-up and the read-outs in
+// double are bound by (1000 x 777 rays: set-up 327 -> 272 us, INVARIANTS 168 ->
+// 158; 524288 single rays: set-up 273 -> 246).
+
+// (double)x
+__device__ __forceinline__ double widen(float x)
+{
+    const unsigned b = __float_as_uint(x), e = b & 0x7f800000u;
+    if (e == 0u || e == 0x7f800000u) // zero, denormal, Inf, NaN
+        return (double)x;
+    return __hiloint2double((int)((b & 0x80000000u) | (((b & 0x7fffffffu) >> 3) + (896u << 20))), (int)(b << 29));
+}
+// (double)k + shift for 0 <= k < 2^32 and a shift of 0 or 1/2: 2^52 + k as it
+// stands in memory, less 2^52 - shift (both exact)
+__device__ __forceinline__ double whole(unsigned k, double shift = 0.0)
+{
+    return __hiloint2double(0x43300000, (int)k) - (4503599627370496.0 - shift);
+}
+// hi = (float)y and lo = (float)((double)hi - y)
+__device__ __forceinline__ void split_pair(double y, float &hi, float &lo)
+{
+    const unsigned hw = (unsigned)__double2hiint(y), lw = (unsigned)__double2loint(y), e = (hw >> 20) & 0x7ffu;
+    if (e - 963u > 120u) { // outside 2^-60 .. 2^61: zero, tiny, huge or not finite
+        hi = (float)y;
+        lo = (float)((double)hi - y);
+        return;
+    }
+    const unsigned rest = lw & 0x1fffffffu; // the 29 bits below single precision
+    unsigned f = (((hw & 0x7fffffffu) << 3) | (lw >> 29)) - (896u << 23);
+    const bool up = rest > 0x10000000u || (rest == 0x10000000u && (f & 1u)); // to nearest, ties to even
+    f += up;
+    hi = __uint_as_float(f | (hw & 0x80000000u));
+    // |hi - y| in units of y's last bit, at most 2^28: two exact halves, one rounding
+    const unsigned d = up ? 0x20000000u - rest : rest;
+    const float a = __uint_as_float(0x4B000000u | (d >> 14)) - 8388608.0f;
+    const float b = __uint_as_float(0x4B000000u | (d & 0x3fffu)) - 8388608.0f;
+    const float v = fmaf(a, 16384.0f, b) * __uint_as_float((e - 948u) << 23);
+    lo = d ? __uint_as_float(__float_as_uint(v) | ((hw & 0x80000000u) ^ (up ? 0u : 0x80000000u))) : 0.0f;
+}
+
 // Workspace of one context (device memory, zeroed before each trace).
 struct Workspace {
     unsigned long long head[4]; // next ray (or list slot) handed out by the queue of each pass
@@ -202,8 +244,9 @@ namespace {
 // --------------------------------------------------------------------------
 
 struct ImageDev {
-    double a, M, r_obs, incl;
-    double si, ci; // sin and cos of incl (host)
+    double a, M, r_obs;
+    float a_lo, M_lo; // low words of a and M: a = (float)a + a_lo
+    double si, ci;    // sin and cos of the inclination (host)
     double a0, da; // Cartesian: alpha of the first pixel edge, pixel width; polar: R0, dR
     double b0, db; // Cartesian: beta likewise; polar: first angle, angle step
     long long first; // first ray of the image relative to the call's first ray
@@ -228,27 +271,28 @@ struct ImageTable {
 
 // Image-plane position of the ray in (row, col) of an image: a pixel centre
 // of the Cartesian grid, or the polar grid point of Sec. 4 (Eqs. 9-10).
-__device__ __forceinline__ void image_point(const ImageDev &im, int64_t row, int64_t col, double &alpha,
+__device__ __forceinline__ void image_point(const ImageDev &im, unsigned row, unsigned col, double &alpha,
                                             double &beta)
 {
     if (im.grid == GRAY_GRID_POLAR) {
-        const double R = im.a0 + ((double)col + 0.5) * im.da;
+        const double R = im.a0 + whole(col, 0.5) * im.da;
         double s, c;
-        sincos(im.b0 + (double)row * im.db, &s, &c);
+        sincos(im.b0 + whole(row) * im.db, &s, &c);
         alpha = R * c;
         beta = R * s;
     } else {
-        alpha = im.a0 + ((double)col + 0.5) * im.da;
-        beta = im.b0 + ((double)row + 0.5) * im.db;
+        alpha = im.a0 + whole(col, 0.5) * im.da;
+        beta = im.b0 + whole(row, 0.5) * im.db;
     }
 }
 
 // Store one initial state (double) into the layout of `prec`.  FP32 modes keep
 // the rounding error of each component in the compensation plane, so a
 // compensated trace starts from the double-precision initial condition.
-// hc: the single-precision constants of (a, M, r_obs), or NULL to compute them.
+// hc: the single-precision constants of (a, M, r_obs), or NULL to compute them;
+// low: the low words of a and M.
 __device__ void store_initial(const StateView &v, int prec, int64_t i, const double *y, double a, double M,
-                              double r_obs, const float *hc)
+                              double r_obs, const float *hc, float2 low)
 {
     if (prec == GRAY_FP64) {
         st_d4(v.X, i, y[0], y[1], y[2], y[3]);
@@ -256,9 +300,11 @@ __device__ void store_initial(const StateView &v, int prec, int64_t i, const dou
         st_d4(v.F, i, y[0], y[1], y[2], y[3]);
     } else {
         float hi[8], lo[8];
+#pragma unroll
         for (int m = 0; m < 8; ++m) {
-            hi[m] = (float)y[m];
-            lo[m] = (prec == GRAY_FP32) ? 0.0f : (float)((double)hi[m] - y[m]);
+            split_pair(y[m], hi[m], lo[m]);
+            if (prec == GRAY_FP32)
+                lo[m] = 0.0f;
         }
         st_f4(v.X, i, hi[0], hi[1], hi[2], hi[3]);
         st_f4(v.K, i, hi[4], hi[5], hi[6], hi[7]);
@@ -277,8 +323,6 @@ __device__ void store_initial(const StateView &v, int prec, int64_t i, const dou
     }
     // the fourth slot of P holds the low words of a and M as two floats
     // (a = (float)a + a_lo): the double-single Eq. 4 test needs them
-    const float a_hi = (float)a, M_hi = (float)M;
-    const float2 low = make_float2((float)(a - (double)a_hi), (float)(M - (double)M_hi));
     double w;
     memcpy(&w, &low, sizeof w);
     st_d4(v.P, i, a, M, r_obs, w);
@@ -315,7 +359,7 @@ __global__ void setup_images_kernel(const __grid_constant__ ImageTable T, int n_
     image_point(im, row, col, alpha, beta);
     double y[8];
     initial_state_sc(im.M, im.a, im.r_obs, im.si, im.ci, alpha, beta, y);
-    store_initial(v, prec, first_ray + i, y, im.a, im.M, im.r_obs, im.hc);
+    store_initial(v, prec, first_ray + i, y, im.a, im.M, im.r_obs, im.hc, make_float2(im.a_lo, im.M_lo));
 }
 
 __global__ void setup_rays_kernel(const double *rays, int64_t n, double M, int64_t first_ray, StateView v, int prec)
@@ -326,7 +370,10 @@ __global__ void setup_rays_kernel(const double *rays, int64_t n, double M, int64
     const double *q = rays + 5 * i;
     double y[8];
     initial_state(M, q[2], q[4], q[3], q[0], q[1], y);
-    store_initial(v, prec, first_ray + i, y, q[2], M, q[4], nullptr);
+    float a_hi, a_lo, M_hi, M_lo;
+    split_pair(q[2], a_hi, a_lo); // the low word of a is a - a_hi, of opposite sign
+    split_pair(M, M_hi, M_lo);
+    store_initial(v, prec, first_ray + i, y, q[2], M, q[4], nullptr, make_float2(-a_lo, -M_lo));
 }
 
 // --------------------------------------------------------------------------
@@ -1613,7 +1660,7 @@ __global__ void probe_rays_kernel(const __grid_constant__ ImageTable T, int n_im
         image_point(im, row, col, alpha, beta);
         double y[8];
         initial_state_sc(im.M, im.a, im.r_obs, im.si, im.ci, alpha, beta, y);
-        store_initial(v, prec, first_ray + i, y, im.a, im.M, im.r_obs, im.hc);
+        store_initial(v, prec, first_ray + i, y, im.a, im.M, im.r_obs, im.hc, make_float2(im.a_lo, im.M_lo));
     }
 }
 
@@ -1728,7 +1775,7 @@ __device__ void load_state_double(const StateView &v, int prec, int64_t i, doubl
         fin[0] = F.x; fin[1] = F.y; fin[2] = F.z; fin[3] = F.w;
     } else {
         const float4 X = ld_f4(v.X, i), K = ld_f4(v.K, i), F = ld_f4(v.F, i);
-        fin[0] = F.x; fin[1] = F.y; fin[2] = F.z; fin[3] = F.w;
+        fin[0] = widen(F.x); fin[1] = widen(F.y); fin[2] = widen(F.z); fin[3] = widen(F.w);
         if (prec == GRAY_FP32_KAHAN_SEL64 && (v.S1[i].w & FLAG_DOUBLE_REPR)) {
             const double2 q0 = ((const double2 *)v.X)[i], q1 = ((const double2 *)v.K)[i];
             const double2 q2 = ((const double2 *)v.CX)[i], q3 = ((const double2 *)v.CK)[i];
@@ -1741,9 +1788,10 @@ __device__ void load_state_double(const StateView &v, int prec, int64_t i, doubl
             CX = ld_f4(v.CX, i);
             CK = ld_f4(v.CK, i);
         }
-        y[0] = (double)X.x - CX.x; y[1] = (double)X.y - CX.y; y[2] = (double)X.z - CX.z; y[3] = (double)X.w - CX.w;
-        y[4] = (double)K.x - CK.x; y[5] = (double)K.y - CK.y; y[6] = (double)K.z - CK.z; y[7] = (double)K.w - CK.w;
-        fin[0] = F.x; fin[1] = F.y; fin[2] = F.z; fin[3] = F.w;
+        y[0] = widen(X.x) - widen(CX.x); y[1] = widen(X.y) - widen(CX.y);
+        y[2] = widen(X.z) - widen(CX.z); y[3] = widen(X.w) - widen(CX.w);
+        y[4] = widen(K.x) - widen(CK.x); y[5] = widen(K.y) - widen(CK.y);
+        y[6] = widen(K.z) - widen(CK.z); y[7] = widen(K.w) - widen(CK.w);
     }
 }
 
@@ -1818,15 +1866,15 @@ __global__ void __launch_bounds__(RECORD_BLOCK) render_record_kernel(StateView v
         load_state_double(v, prec, i, y, fin);
         const int4 s0 = v.S0[i];
         double *o = rows + 17 * threadIdx.x;
-        o[0] = s0.x;
-        o[1] = s0.y;
-        o[2] = s0.z;
-        o[3] = s0.w;
+        o[0] = whole((unsigned)s0.x); // status and counts are never negative
+        o[1] = whole((unsigned)s0.y);
+        o[2] = whole((unsigned)s0.z);
+        o[3] = whole((unsigned)s0.w);
         for (int m = 0; m < 4; ++m)
             o[4 + m] = fin[m];
         for (int m = 0; m < 8; ++m)
             o[8 + m] = y[m];
-        o[16] = v.S1[i].x;
+        o[16] = whole((unsigned)v.S1[i].x);
     }
     __syncthreads();
     const int count = 17 * (int)(n - j0 < RECORD_BLOCK ? n - j0 : RECORD_BLOCK);
@@ -1835,7 +1883,7 @@ __global__ void __launch_bounds__(RECORD_BLOCK) render_record_kernel(StateView v
 }
 
 // GRAY_RENDER_INVARIANTS, in double from the stored state (bound by the FP64
-// pipe: a sine and cosine, a square root and four divides per ray).
+// pipe: a sine and cosine, a square root and three reciprocals per ray).
 __global__ void render_invariants_kernel(StateView v, int prec, int64_t first, int64_t n, double *out)
 {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -1848,13 +1896,18 @@ __global__ void render_invariants_kernel(StateView v, int prec, int64_t first, i
     const Hole<double> H = make_hole(p.x, p.y, p.z, 1.0, 1.0, 0.0);
     double s, c;
     sincos(y[2], &s, &c);
-    const MetricPieces<double> m = metric_pieces(H, y[1], s, c);
+    // the metric of metric_pieces, with refined reciprocals for its divides
+    const double r = y[1], a2 = H.a * H.a, s2 = s * s;
+    const double Sigma = fma(a2, c * c, r * r), iS = recip(Sigma);
+    const double u = 2.0 * H.M * r * iS;
+    const double gtt = u - 1.0, gtp = -u * H.a * s2, gpp = (fma(r, r, a2) + u * a2 * s2) * s2;
+    const double grr = Sigma * recip(fma(r - H.rp, r - H.rm, H.dc));
     const double kt = y[4], kr = y[5], kh = y[6], kp = y[7];
-    const double E = -(m.gtt * kt + m.gtp * kp);
-    const double L = m.gtp * kt + m.gpp * kp;
-    const double kth_low = m.gthth * kh;
-    const double Q = kth_low * kth_low + c * c * (-H.a * H.a * E * E + L * L / (s * s));
-    const double N = m.gtt * kt * kt + 2.0 * m.gtp * kt * kp + m.grr * kr * kr + m.gthth * kh * kh + m.gpp * kp * kp;
+    const double E = -(gtt * kt + gtp * kp);
+    const double L = gtp * kt + gpp * kp;
+    const double kth_low = Sigma * kh;
+    const double Q = kth_low * kth_low + c * c * (-H.a * H.a * E * E + L * L * recip(s2));
+    const double N = gtt * kt * kt + 2.0 * gtp * kt * kp + grr * kr * kr + Sigma * kh * kh + gpp * kp * kp;
     double *o = out + 4 * j;
     o[0] = E;
     o[1] = L;
@@ -2539,7 +2592,8 @@ ImageDev image_dev(const gray_image &im, int64_t first)
     d.a = im.a;
     d.M = im.M;
     d.r_obs = im.r_obs;
-    d.incl = im.incl;
+    d.a_lo = (float)(im.a - (double)(float)im.a);
+    d.M_lo = (float)(im.M - (double)(float)im.M);
     d.si = std::sin(im.incl);
     d.ci = std::cos(im.incl);
     d.a0 = im.alpha0;
