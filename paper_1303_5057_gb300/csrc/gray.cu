@@ -3074,19 +3074,22 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
                 cudaEventRecord(ctx->ev[2], s);
                 ctx->ev_used[1] = true;
             }
-            // one block per SM: the double pipe is shared by the SM and a warp
-            // instruction holds it whatever its active lanes, so few warps,
-            // each draining many zone rays, waste the fewest pipe cycles on
-            // partly filled warps (measured: 1.95 ms at three blocks per SM,
-            // 1.53 ms at one, 2.2 ms with 64-thread blocks)
-            if (ctx->opt.zone_arith == GRAY_ZONE_FP64)
+            // IEEE double: one block per SM.  The double pipe is shared by
+            // the SM and a warp instruction holds it whatever its active
+            // lanes, so few warps, each draining many zone rays, waste the
+            // fewest pipe cycles on partly filled warps (1.95 ms at three
+            // blocks per SM, 1.53 ms at one, 2.2 ms with 64-thread blocks).
+            // Double-single: two blocks per SM, which hide each other's
+            // refills and instruction fetches (1024^2 image 0.319 ms at one,
+            // 0.276 at two, 0.329 at three; r_sw = 0.25: 2.26 / 2.07 / 2.33;
+            // 524288 mixed rays 0.69 / 0.555 / 0.64).
+            if (ctx->opt.zone_arith == GRAY_ZONE_FP64) {
                 zone_kernel<true, double><<<(unsigned)ctx->num_sms, block, 0, s>>>(Z);
-            else
-            {
-                const auto kernel = Z.stop_equator ? zone_kernel<true, ds, CFG_EQUATOR>
+            } else {
+                const auto kernel = Z.stop_equator                     ? zone_kernel<true, ds, CFG_EQUATOR>
                                     : Z.step_rule == GRAY_STEP_EQ2 ? zone_kernel<true, ds, CFG_EQ2>
-                                                                   : zone_kernel<true, ds, CFG_BENCH>;
-                kernel<<<(unsigned)ctx->num_sms, block, 0, s>>>(Z);
+                                                                       : zone_kernel<true, ds, CFG_BENCH>;
+                kernel<<<2u * (unsigned)ctx->num_sms, block, 0, s>>>(Z);
             }
             if ((rc = check_launch()))
                 return rc;
