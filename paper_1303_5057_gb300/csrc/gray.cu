@@ -526,7 +526,7 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
     if constexpr (sizeof(T) == 4 && KAHAN) {
         bool ambiguous;
         redo = xi_fails_flag(H, g1, y1, O.eps_xi, ambiguous);
-        if (ambiguous && aM_lo) {
+        if (rarely(ambiguous && aM_lo)) {
             const float2 lo = *aM_lo;
             redo = xi_fails_ds(y1, c1, make_float4(H.a, lo.x, H.M, lo.y), O.eps_xi);
         }
@@ -554,7 +554,7 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
     // behind one test, so a plain step takes a single branch here.
     const T half_pi = T(0.5) * pi_v<T>();
     const bool equator = O.stop_equator && (y[2] - half_pi) * (y1[2] - half_pi) < T(0);
-    if (!finite || equator || y1[1] <= H.r_cap || y1[1] >= H.r_esc || y1[2] > pi_v<T>() || y1[2] < T(0)) {
+    if (rarely(!finite || equator || y1[1] <= H.r_cap || y1[1] >= H.r_esc || y1[2] > pi_v<T>() || y1[2] < T(0))) {
         // the out-of-line helpers get copies made here: only these copies
         // have their address taken, so the step's states stay in registers
         // (without them the pass stored ~6 words to local memory per warp
@@ -860,7 +860,7 @@ __global__ void __maxnreg__(MAXREG) trace32_kernel(TraceArgs A)
             if (has) {
                 int status = GRAY_RAY_ACTIVE;
                 bool yield = false;
-                if (steps >= stop_at || (SEL64 && y[1] - c[1] < r_promote) || stop) {
+                if (rarely(steps >= stop_at || (SEL64 && y[1] - c[1] < r_promote) || stop)) {
                     if (steps >= A.max_steps) {
                         status = GRAY_RAY_STEP_CAP;
                         for (int m = 0; m < 4; ++m)
@@ -874,7 +874,7 @@ __global__ void __maxnreg__(MAXREG) trace32_kernel(TraceArgs A)
                     status = step_once<float, KAHAN>(H, O, y, c, geo, fin, euler, remaps, (const float2 *)&v.P[id].w);
                     ++steps;
                 }
-                if (status != GRAY_RAY_ACTIVE || yield || handoff) {
+                if (rarely(status != GRAY_RAY_ACTIVE || yield || handoff)) {
                     st_f4(v.X, id, y[0], y[1], y[2], y[3]);
                     st_f4(v.K, id, y[4], y[5], y[6], y[7]);
                     if (KAHAN) {
