@@ -1217,6 +1217,19 @@ template <typename T> __device__ __forceinline__ void load_zone_state(const Stat
     }
 }
 
+// Steps after a warp found the list drained before the block's last rays may
+// go to a team: the rays of the benchmark rule are done by then (at most ~20
+// zone steps each).
+constexpr int ZONE_TAIL = 32;
+
+// Four warps of a block as a team on 32 zone rays (zone_team).
+struct TeamShared {
+    float2 v[2][8][32]; // exchanged values, two buffers so that one barrier per exchange is enough
+    int active[4], go;  // hand-over from zone_lanes: rays left per warp, and its start
+    int listed, id[32]; // the rays handed over
+    int stop;           // the context was cancelled
+};
+
 // Zone kernel of GRAY_FP32_KAHAN_SEL64: the rays of the hand-off list, in
 // extended precision T (double, or double-single on the single-precision
 // pipe: GRAY_ZONE_DS) while r < r_demote (= r_promote + r_sw).  RETURN = true
@@ -1229,12 +1242,17 @@ template <typename T> __device__ __forceinline__ void load_zone_state(const Stat
 // The switches are exact one way (hi - lo to T) and a rounding the other way
 // (T to hi, lo; exact for double-single), the same in both forms, so a ray's
 // arithmetic does not depend on which pass runs it.
-template <bool RETURN, typename T, int CFG = CFG_EQUATOR>
-__global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
+//
+// TEAM (double-single, first pass): once the list is drained and no more rays
+// are left in the block than a team holds, the warps list them in `sh` and
+// return, for zone_team to finish.
+template <bool RETURN, typename T, int CFG, bool TEAM>
+__device__ __forceinline__ void zone_lanes(const TraceArgs &A, TeamShared *sh)
 {
     using Z = ZoneArith<T>;
     const unsigned FULL = 0xffffffffu;
     const int lane = threadIdx.x & 31;
+    int drained = 0; // TEAM: steps since the list was drained
     const StateView &v = A.v;
     StepOpt<T> Od;
     Od.h_frac = T(A.h_frac);
@@ -1315,8 +1333,46 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
             if ((int64_t)base + cnt >= n)
                 exhausted = true;
         }
-        if (!__any_sync(FULL, has))
+        if constexpr (TEAM) {
+            bool go = false;
+            if (exhausted && ++drained > ZONE_TAIL) {
+                const int mine = __popc(__ballot_sync(FULL, has));
+                if (lane == 0) {
+                    volatile int *active = sh->active;
+                    active[threadIdx.x >> 5] = mine;
+                    if (active[0] + active[1] + active[2] + active[3] <= 32)
+                        *(volatile int *)&sh->go = 1;
+                    go = *(volatile int *)&sh->go != 0;
+                }
+                go = __shfl_sync(FULL, (int)go, 0) != 0;
+            }
+            if (go) {
+                const unsigned left = __ballot_sync(FULL, has);
+                int base = 0;
+                if (lane == 0)
+                    base = atomicAdd(&sh->listed, __popc(left));
+                base = __shfl_sync(FULL, base, 0);
+                if (has) {
+                    sh->id[base + __popc(left & ((1u << lane) - 1u))] = (int)id;
+                    float hi[8], lo[8];
+#pragma unroll
+                    for (int m = 0; m < 8; ++m)
+                        Z::to_pair(yd[m], hi[m], lo[m]);
+                    st_f4(v.X, id, hi[0], hi[1], hi[2], hi[3]);
+                    st_f4(v.K, id, hi[4], hi[5], hi[6], hi[7]);
+                    st_f4(v.CX, id, lo[0], lo[1], lo[2], lo[3]);
+                    st_f4(v.CK, id, lo[4], lo[5], lo[6], lo[7]);
+                    v.S0[id] = make_int4(GRAY_RAY_ACTIVE, steps, euler, remaps);
+                    v.S1[id] = make_int4(n64, epoch, used, FLAG_DOUBLE_MODE);
+                }
+                break;
+            }
+        }
+        if (!__any_sync(FULL, has)) {
+            if (TEAM && lane == 0)
+                ((volatile int *)sh->active)[threadIdx.x >> 5] = 0;
             break;
+        }
 
         for (int k = 0; k < A.refill; ++k) {
             bool ret = false; // this lane's ray climbed out and goes to the return list
@@ -1422,6 +1478,260 @@ __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(TraceArgs A)
         }
     }
     warp_stats<double>(A, lane, tot_steps, tot_euler, tot_fp64, true);
+}
+
+// One component of the acceleration (accel_geo's expressions; the other
+// components' operations fall away).  w is uniform over the warp.
+__device__ __forceinline__ ds accel_component(const Hole<ds> &H, const Geo<ds> &g, int w, ds kt, ds kr, ds kh, ds kp)
+{
+    ds a[4];
+    if (w == 0) {
+        accel_geo(H, g, kt, kr, kh, kp, a);
+        return a[0];
+    }
+    if (w == 1) {
+        accel_geo(H, g, kt, kr, kh, kp, a);
+        return a[1];
+    }
+    if (w == 2) {
+        accel_geo(H, g, kt, kr, kh, kp, a);
+        return a[2];
+    }
+    accel_geo(H, g, kt, kr, kh, kp, a);
+    return a[3];
+}
+
+// The last zone rays of a block, four warps per 32 rays.  A double-single step
+// is ~3700 instructions in one warp, 5.5 us when the warp is alone, and under
+// Eq. 2 a ray near a pole takes up to a thousand zone steps where the others
+// take 40: that one ray was the pass.  Here lane l of each of the block's four
+// warps holds ray l; warp w computes component w of every acceleration and of
+// the RK4 sums (half of a step's work) on its own scheduler, and the warps
+// exchange the stage's momentum through shared memory, one barrier per stage:
+// 4.5 us a step.  The geometry, the Eq. 4 test and every decision are formed by
+// all four warps alike, so control flow is the same in each; warp w stores its
+// share of a finished ray.  Operations and results are those of zone_lanes.
+template <int CFG> __device__ __noinline__ void zone_team(const TraceArgs &A, TeamShared &sh)
+{
+    const unsigned FULL = 0xffffffffu;
+    const int lane = threadIdx.x & 31, w = __shfl_sync(FULL, threadIdx.x >> 5, 0);
+    const StateView &v = A.v;
+    StepOpt<ds> O;
+    O.h_frac = ds(A.h_frac);
+    O.h_min = ds(A.h_min);
+    O.eps_xi = ds(A.eps_xi);
+    O.step_rule = CFG == CFG_EQUATOR ? A.step_rule : CFG == CFG_EQ2 ? GRAY_STEP_EQ2 : GRAY_STEP_BENCH;
+    O.stop_equator = CFG == CFG_EQUATOR ? A.stop_equator : 0;
+    const int epoch = *A.epoch_dev;
+    const ds r_sw = ds(A.r_sw), cap_frac = ds(A.cap_frac), r_esc_frac = ds(A.r_esc_frac);
+
+    bool has = false;
+    int64_t id = 0;
+    ds y[8], cz[8];
+    Hole<ds> H = make_hole_ds(make_float4(0.0f, 0.0f, 0.0f, 0.0f), make_float4(0.0f, 0.0f, 0.0f, 1000.0f),
+                              make_float2(0.0f, 0.0f), cap_frac, r_esc_frac, r_sw);
+    Geo<ds> g;
+    ds r_demote = ds(INFINITY);
+    int steps = 0, euler = 0, remaps = 0, n64 = 0, used = 0;
+    unsigned long long tot_steps = 0, tot_euler = 0;
+#pragma unroll
+    for (int m = 0; m < 8; ++m) {
+        cz[m] = ds(0.0);
+        y[m] = ds(m == 1 ? 10.0 : m == 2 ? 1.0 : 0.0); // idle lanes: a photon at rest
+    }
+    g = geometry(H, y[1], y[2]);
+    int buf = 0;
+
+    const int my = lane < sh.listed ? sh.id[lane] : -1;
+    if (my >= 0) {
+        const int4 s0 = v.S0[my], s1 = v.S1[my];
+        has = true;
+        id = my;
+        steps = s0.y;
+        euler = s0.z;
+        remaps = s0.w;
+        n64 = s1.x;
+        used = s1.z;
+        H = make_hole_ds(v.PF0[my], v.PF1[my], *(const float2 *)&v.P[my].w, cap_frac, r_esc_frac, r_sw);
+        r_demote = H.r_promote + r_sw;
+        load_zone_state(v, my, s1.w, y);
+        g = geometry(H, y[1], y[2]);
+    }
+
+    while (__any_sync(FULL, has)) { // the same in every warp
+        // gray_cancel, as in trace32_kernel (the barriers of the last step
+        // lie between its reads of sh.stop and this write)
+        if (w == 0) {
+            const bool stop = cancelled(A, lane);
+            if (lane == 0)
+                sh.stop = stop;
+        }
+        __syncthreads();
+        const bool stop = sh.stop != 0;
+
+        // ---- one step of every lane that takes one ----
+        const bool capped = has && steps >= A.max_steps;
+        const bool yield = has && !capped && (stop || (A.budget > 0 && used >= A.budget));
+        const bool ret = has && !capped && !yield && y[1] >= r_demote; // climbs out of the zone
+        const bool live = has && !capped && !yield && !ret;
+        ds h = step_size(H, O, y);
+        const ds hh = scaled(h, 0.5), h6 = sixth(h);
+        ds a1;
+        {
+            ds a = accel_component(H, g, w, y[4], y[5], y[6], y[7]);
+            a1 = a;
+            ds pk[4] = {y[4], y[5], y[6], y[7]}, pa = a, yk = w == 0 ? y[4] : w == 1 ? y[5] : w == 2 ? y[6] : y[7];
+            ds sk = yk, sa = a;
+            const ds yx = w == 0 ? y[0] : w == 1 ? y[1] : w == 2 ? y[2] : y[3];
+#pragma unroll 1
+            for (int stage = 0; stage < 3; ++stage) {
+                const ds cs = stage < 2 ? hh : h;
+                const float wt = stage < 2 ? 2.0f : 1.0f;
+                const ds ks = fma(cs, pa, yk);
+                sh.v[buf][w][lane] = make_float2(ks.hi, ks.lo);
+                const ds rs = fma(cs, pk[1], y[1]), ths = fma(cs, pk[2], y[2]);
+                const Geo<ds> gs = geometry_rel(H, g, rs, cs * pk[2], ths, ds(0.0), ds(0.0));
+                __syncthreads();
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float2 e = sh.v[buf][m][lane];
+                    pk[m] = ds{e.x, e.y};
+                }
+                buf ^= 1;
+                pa = accel_component(H, gs, w, pk[0], pk[1], pk[2], pk[3]);
+                sk = fma_scaled(ks, wt, sk);
+                sa = fma_scaled(pa, wt, sa);
+            }
+            const ds xn = yx + h6 * sk, kn = yk + h6 * sa;
+            sh.v[buf][w][lane] = make_float2(xn.hi, xn.lo);
+            sh.v[buf][4 + w][lane] = make_float2(kn.hi, kn.lo);
+            sh.v[buf ^ 1][4 + w][lane] = make_float2(a1.hi, a1.lo); // for an Euler redo
+        }
+        __syncthreads();
+        ds y1[8];
+#pragma unroll
+        for (int m = 0; m < 8; ++m) {
+            const float2 e = sh.v[buf][m][lane];
+            y1[m] = ds{e.x, e.y};
+        }
+        Geo<ds> g1 = geometry(H, y1[1], y1[2]);
+        int status = GRAY_RAY_ACTIVE;
+        ds fin[4];
+        if (live) {
+            if (xi_fails(H, g1, y1, O.eps_xi)) { // forward Euler at h/9
+                h = ninth(h);
+#pragma unroll
+                for (int m = 0; m < 4; ++m) {
+                    const float2 e = sh.v[buf ^ 1][4 + m][lane];
+                    y1[m] = y[m] + h * y[4 + m];
+                    y1[4 + m] = y[4 + m] + h * ds{e.x, e.y};
+                }
+                g1 = geometry(H, y1[1], y1[2]);
+                ++euler;
+                ++tot_euler;
+            }
+            bool finite = true;
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+                finite &= finite_v(y1[m]);
+            const ds half_pi = ds(0.5) * pi_v<ds>();
+            const bool equator = O.stop_equator && (y[2] - half_pi) * (y1[2] - half_pi) < ds(0.0);
+            if (!finite || equator || y1[1] <= H.r_cap || y1[1] >= H.r_esc || y1[2] > pi_v<ds>() || y1[2] < ds(0.0)) {
+                ds s0[8], s1[8], sf[4];
+#pragma unroll
+                for (int m = 0; m < 8; ++m) {
+                    s0[m] = y[m];
+                    s1[m] = y1[m];
+                }
+                const bool out = y1[1] >= H.r_esc && h * y1[5] > ds(0.0);
+                status = !finite ? GRAY_RAY_NONFINITE : equator ? GRAY_RAY_EQUATOR : y1[1] <= H.r_cap
+                         ? GRAY_RAY_CAPTURED : out ? GRAY_RAY_ESCAPED : GRAY_RAY_ACTIVE;
+                if (w == 3 && status != GRAY_RAY_ACTIVE) { // the warp that stores the stop point
+                    if (status == GRAY_RAY_NONFINITE) {
+                        for (int m = 0; m < 4; ++m)
+                            sf[m] = y1[m];
+                    } else if (status == GRAY_RAY_EQUATOR) {
+                        equator_crossing(s0, s1, h, sf);
+                    } else {
+                        stop_surface_mixed(s0, s1, h, status == GRAY_RAY_CAPTURED ? H.r_cap : H.r_esc, sf);
+                    }
+#pragma unroll
+                    for (int m = 0; m < 4; ++m)
+                        fin[m] = sf[m];
+                }
+                if (status != GRAY_RAY_NONFINITE && remap_eq3<ds, false>(y1, cz)) {
+                    ++remaps;
+                    g1 = geometry(H, y1[1], y1[2]);
+                }
+            }
+#pragma unroll
+            for (int m = 0; m < 8; ++m)
+                y[m] = y1[m];
+            g = g1;
+            ++n64;
+            ++steps;
+            ++used;
+            ++tot_steps;
+        }
+        if (capped) {
+            status = GRAY_RAY_STEP_CAP;
+#pragma unroll
+            for (int m = 0; m < 4; ++m)
+                fin[m] = y[m];
+        }
+        if (has && (status != GRAY_RAY_ACTIVE || yield || ret)) {
+            // a double-single state is a compensated pair
+            if (w == 0)
+                st_f4(v.X, id, y[0].hi, y[1].hi, y[2].hi, y[3].hi);
+            if (w == 1)
+                st_f4(v.K, id, y[4].hi, y[5].hi, y[6].hi, y[7].hi);
+            if (w == 2) {
+                st_f4(v.CX, id, -y[0].lo, -y[1].lo, -y[2].lo, -y[3].lo);
+                st_f4(v.CK, id, -y[4].lo, -y[5].lo, -y[6].lo, -y[7].lo);
+            }
+            if (w == 3) {
+                if (status != GRAY_RAY_ACTIVE)
+                    st_f4(v.F, id, fin[0].hi, fin[1].hi, fin[2].hi, fin[3].hi);
+                v.S0[id] = make_int4(status, steps, euler, remaps);
+                v.S1[id] = make_int4(n64, epoch, used, yield ? FLAG_DOUBLE_MODE : 0);
+            }
+            has = false;
+        }
+        if (w == 0) {
+            int rank;
+            const unsigned long long rb = warp_count(&A.ws->demoted, ret, lane, &rank);
+            if (ret)
+                v.R[rb + rank] = (int)id;
+        }
+        buf ^= 1; // the next exchange writes the buffer that no warp reads any more
+    }
+    if (w == 0)
+        warp_stats<double>(A, lane, tot_steps, tot_euler, tot_steps, true);
+}
+
+// The zone kernels.  The double-single first pass ends with teams: with the
+// four warps' code in the instruction cache at once a team loses to a ray per
+// lane on short rests (1024^2 image 0.276 -> 0.35 ms when every block's last 32
+// rays went to teams), so the hand-over waits for ZONE_TAIL steps after the
+// list is drained.  Eq. 2 image, 509^2: zone pass 5.35 -> 4.35 ms
+// (24 and 48 steps the same within its runs).
+template <bool RETURN, typename T, int CFG = CFG_EQUATOR>
+__global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(const __grid_constant__ TraceArgs A)
+{
+    if constexpr (RETURN && std::is_same<T, ds>::value) {
+        __shared__ TeamShared sh;
+        if (threadIdx.x < 4)
+            sh.active[threadIdx.x] = 1000; // not drained yet
+        if (threadIdx.x == 0)
+            sh.go = sh.listed = 0;
+        __syncthreads();
+        zone_lanes<RETURN, T, CFG, true>(A, &sh);
+        __syncthreads();
+        if (sh.listed)
+            zone_team<CFG>(A, sh);
+    } else {
+        zone_lanes<RETURN, T, CFG, false>(A, nullptr);
+    }
 }
 
 // The queue of a trace without a caller's order: the ACTIVE rays, those that
