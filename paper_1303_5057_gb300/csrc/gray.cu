@@ -3246,24 +3246,29 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
 // A double-precision pass.  An SM takes one FP64 instruction per 19 cycles and
 // a warp at most one per 64, so four warps fill the pipe; more only slow each
 // other down, and the longest rays with them.  Warps are single blocks, spread
-// evenly over the SMs, W64_PER_SM = 5 to an SM.  (300 x 211 image, a = 0.9,
-// i = 75 deg, planned: three 128-thread blocks per SM 107 ms, 4 / 5 / 6 / 8
-// warps 60 / 66 / 74 / 90 ms; 512^2: 136 ms, then 109 / 108 / 108 / 115;
-// 1024 x 640: 253 ms, then 251 / 250 / 250 / 250.)
+// evenly over the SMs, four to an SM; a queue long enough that its last rays
+// do not matter takes five (300 x 211 image, a = 0.9, i = 75 deg, planned:
+// three 128-thread blocks per SM 107 ms, 3 / 4 / 5 / 6 / 8 warps 58 / 60 / 66 /
+// 74 / 90; with the hand-over below 49.4 / 49.5 / 51.1 ms at 3 / 4 / 5; 512 x
+// 400: 97 / 82 / 86; 1024^2: 471 / 395 / 392).
 //
 // Up to QUAD_RAYS_PER_SM rays per SM go to the four-lane kernel at once: there
 // a step of one ray takes 12.7 us instead of 19 (64^2: 45 -> 29 ms; 128^2
-// planned: 60 -> 42), while a chip full of rays does 1.7 times the steps per
-// second with a ray per lane (1024 x 640: 250 ms against 433; 300 x 211
-// planned is the crossover: 60 against 51 ms, under Eq. 2 48 against 70).  In
+// planned: 60 -> 42; 170 x 150: 39 against 42 from the one-lane kernel), while
+// a chip full of rays does 1.7 times the steps per second with a ray per lane
+// (1024 x 640: 250 ms against 433; 300 x 211 under Eq. 2 48 against 70).  In
 // longer queues the one-lane kernel hands its last rays over (A.handover;
-// 300 x 211: 66 -> 54 ms planned, 62 -> 51 in natural order, 48 -> 44 Eq. 2).
-constexpr int W64_PER_SM = 5, QUAD_PER_SM = 6, QUAD_RAYS_PER_SM = 160, QUAD_HANDOVER_PER_SM = 32;
+// 300 x 211 natural order 62 -> 51, Eq. 2 48 -> 44; 16 to 64 rays per SM are
+// within 2 % of each other).
+constexpr int W64_PER_SM = 4, W64_PER_SM_LONG = 5, LONG_RAYS_PER_SM = 2048;
+constexpr int QUAD_PER_SM = 6, QUAD_RAYS_PER_SM = 200, QUAD_HANDOVER_PER_SM = 32;
 
 int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
 {
     const int64_t sms = ctx->num_sms;
-    int64_t per_sm = ctx->opt.blocks_per_sm > 0 ? 4 * (int64_t)ctx->opt.blocks_per_sm : W64_PER_SM;
+    int64_t per_sm = ctx->opt.blocks_per_sm > 0       ? 4 * (int64_t)ctx->opt.blocks_per_sm
+                     : work > LONG_RAYS_PER_SM * sms ? W64_PER_SM_LONG
+                                                     : W64_PER_SM;
     int64_t quad_work = work;
     if (work > QUAD_RAYS_PER_SM * sms) {
         A.handover = std::min(QUAD_HANDOVER_PER_SM * sms, A.n); // the list holds n entries

@@ -1,6 +1,6 @@
 """Double precision with four lanes per ray against one ray per lane.
 
-Queues of up to 160 rays per SM are traced by the four-lane kernel, longer ones
+Queues of up to 200 rays per SM are traced by the four-lane kernel, longer ones
 by the one-lane kernel, whose last rays the four-lane kernel takes over.  Both
 do the same operations on the same operands, so a ray's record is the same
 bits in each (no tolerance): an image alone, and as many copies of it in one
@@ -48,7 +48,7 @@ def test_four_lanes_per_ray_give_the_bits_of_one(name, budgets):
     im, options = CASES[name]
     opt = gray.Options(precision=gray.FP64, **{"max_steps": 20000, **options})
     alone = records([im], opt, budgets)
-    limit = 160 * torch.cuda.get_device_properties(0).multi_processor_count
+    limit = 200 * torch.cuda.get_device_properties(0).multi_processor_count
     copies = limit // im.n + 1
     many = records([im] * copies, opt, budgets).reshape(copies, im.n, -1)
     assert np.all(alone[:, 0] != gray.ACTIVE)
@@ -62,7 +62,7 @@ def test_a_short_state_with_a_long_queue_keeps_its_hand_off_list():
     im = I.Image(a=0.9, incl=1.0, nx=9, ny=7)
     opt = gray.Options(precision=gray.FP64, max_steps=20000)
     want = records([im], opt, (0,))
-    limit = 160 * torch.cuda.get_device_properties(0).multi_processor_count
+    limit = 200 * torch.cuda.get_device_properties(0).multi_processor_count
     order = torch.full((limit + 100,), -1, dtype=torch.int32, device="cuda")
     order[50:50 + im.n] = torch.arange(im.n, dtype=torch.int32, device="cuda")
     tr = gray.Tracer(opt, im.n)
