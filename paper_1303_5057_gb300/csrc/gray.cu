@@ -3195,11 +3195,15 @@ unsigned persistent_grid(const gray_ctx *ctx, const void *kernel, int block, int
     return (unsigned)(want > 0 ? want : 1);
 }
 
-// Rays that a single-precision pass holds at once (its kernel keeps four
-// blocks of 128 threads on an SM), and the step budget below which a pass ends
-// too soon for its queue's order to matter.
+// A trace without an order makes a lead-first queue of more than 1.6 times the
+// rays that the pass holds at once (four blocks of 128 threads on an SM).  With
+// fewer, most rays start at once in any order, and warps full of crawling rays
+// only crawl together (medians of 23 runs, three holes: 300^2 images 3.5 ms
+// ordered, 3.1 in natural order; 340^2 3.35 and 3.44; 370^2 3.48 and 3.60;
+// 400^2 3.61 and 3.77; 180000 mixed rays 4.7 and 5.3).  Nor under a step
+// budget that ends the pass too soon for its queue's order to matter.
 constexpr int ORDER_MIN_BUDGET = 512;
-int64_t resident_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512; }
+int64_t order_min_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512 * 8 / 5; }
 
 // One single- or double-precision pass over the queue of A (no zone kernel).
 // A persistent single-precision pass.  A queue of up to three blocks per SM
@@ -3352,9 +3356,7 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             cudaEventRecord(ctx->ev[0], s);
             ctx->ev_used[0] = true;
         }
-        // more rays than the pass holds at once and no budget that ends it
-        // early: the order of the queue decides when its last ray ends
-        if (!order && ctx->opt.precision != GRAY_FP64 && !A.one_per_thread && n_state > resident_rays(ctx) &&
+        if (!order && ctx->opt.precision != GRAY_FP64 && !A.one_per_thread && n_state > order_min_rays(ctx) &&
             (step_budget <= 0 || step_budget > ORDER_MIN_BUDGET)) {
             int *list = A.v.R ? A.v.R : A.v.L; // the zone pass fills R later; the other modes leave L unused
             order_rays_kernel<<<grid_for(n_state, ORDER_RAYS), ORDER_BLOCK, 0, s>>>(A.v, n_state, list, ctx->ws);

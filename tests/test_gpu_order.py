@@ -1,7 +1,7 @@
 """The lead-first queue of a trace without a caller's order.
 
-A trace of more rays than the single-precision pass holds at once (512 per SM)
-orders its ACTIVE rays itself; a ray's result does not depend on its place in
+A trace of more than 1.6 times the rays that the single-precision pass holds at
+once (512 per SM) orders its ACTIVE rays itself; a ray's result does not depend on its place in
 the queue, so every record equals, bit for bit (no tolerance), that of the
 same trace under an explicit order."""
 import math
@@ -30,7 +30,7 @@ def trace(opt, n, prepare, budgets, order):
 @pytest.mark.parametrize("extra", [1, 1023, 5000])
 @pytest.mark.parametrize("precision", ["fp32", "fp32_kahan", "fp32_kahan_sel64"])
 def test_lead_first_queue_equals_an_explicit_order(precision, extra):
-    n = 512 * torch.cuda.get_device_properties(0).multi_processor_count + extra
+    n = 512 * 8 * torch.cuda.get_device_properties(0).multi_processor_count // 5 + extra
     opt = gray.Options(precision=gray.PRECISIONS[precision], max_steps=20000, r_sw=0.02)
     rays = torch.from_numpy(I.mixed_rays(n, offset=11 * n)).cuda()
 
@@ -49,7 +49,7 @@ def test_lead_first_queue_of_a_resumed_trace(image):
     """All rays in one class (M = 0: none leads; face-on: L_z = 0, all lead),
     most of them finished when the second call orders what is left."""
     sms = torch.cuda.get_device_properties(0).multi_processor_count
-    side = int(math.isqrt(512 * sms)) + 3
+    side = int(math.isqrt(512 * 8 * sms // 5)) + 3
     im = I.Image(a=0.3, M=0.0, incl=1.0, nx=side, ny=side) if image == "flat" else \
         I.Image(a=0.9, incl=0.0, nx=side, ny=side)
     opt = gray.Options(precision=gray.FP32_KAHAN_SEL64, max_steps=20000, r_sw=0.02, step_rule=gray.STEP_EQ2)
