@@ -3256,16 +3256,21 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
 // 74 / 90; with the hand-over below 49.4 / 49.5 / 51.1 ms at 3 / 4 / 5; 512 x
 // 400: 97 / 82 / 86; 1024^2: 471 / 395 / 392).
 //
-// Up to QUAD_RAYS_PER_SM rays per SM go to the four-lane kernel at once: there
-// a step of one ray takes 12.7 us instead of 19 (64^2: 45 -> 29 ms; 128^2
-// planned: 60 -> 42; 170 x 150: 39 against 42 from the one-lane kernel), while
-// a chip full of rays does 1.7 times the steps per second with a ray per lane
-// (1024 x 640: 250 ms against 433; 300 x 211 under Eq. 2 48 against 70).  In
-// longer queues the one-lane kernel hands its last rays over (A.handover;
-// 300 x 211 natural order 62 -> 51, Eq. 2 48 -> 44; 16 to 64 rays per SM are
-// within 2 % of each other).
+// Short queues go to the four-lane kernel at once: there a step of one ray
+// takes 12.7 us instead of 19 (64^2: 45 -> 29 ms), while a chip full of rays
+// does 1.7 times the steps per second with a ray per lane (1024 x 640: 250 ms
+// against 433).  How many rays are few depends on how far the longest exceed
+// the others: under the benchmark rule a planned queue is bound by its long
+// rays up to 200 rays per SM (158^2: 41.7 ms, 43.6 from the one-lane kernel;
+// 170 x 150: 39 and 42), one in any order up to 80 (100^2: 31.1 and 32.8, but
+// 140^2: 42.7 and 38.5); under Eq. 2, whose rays are alike, up to 64 (80^2: 12.0
+// and 15.3, but 120^2: 21.1 and 17.1, 158^2: 27.0 and 19.1).  In longer queues
+// the one-lane kernel hands its last rays over (A.handover; 300 x 211 natural
+// order 62 -> 51, Eq. 2 48 -> 44; 16 to 64 rays per SM are within 2 % of each
+// other).
 constexpr int W64_PER_SM = 4, W64_PER_SM_LONG = 5, LONG_RAYS_PER_SM = 2048;
-constexpr int QUAD_PER_SM = 6, QUAD_RAYS_PER_SM = 200, QUAD_HANDOVER_PER_SM = 32;
+constexpr int QUAD_PER_SM = 6, QUAD_HANDOVER_PER_SM = 32;
+constexpr int QUAD_RAYS_PLANNED = 200, QUAD_RAYS_ANY_ORDER = 80, QUAD_RAYS_EQ2 = 64; // per SM
 
 int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
 {
@@ -3274,7 +3279,10 @@ int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
                      : work > LONG_RAYS_PER_SM * sms ? W64_PER_SM_LONG
                                                      : W64_PER_SM;
     int64_t quad_work = work;
-    if (work > QUAD_RAYS_PER_SM * sms) {
+    const int quad_rays = A.step_rule == GRAY_STEP_EQ2 ? QUAD_RAYS_EQ2
+                          : A.order                    ? QUAD_RAYS_PLANNED
+                                                       : QUAD_RAYS_ANY_ORDER;
+    if (work > quad_rays * sms) {
         A.handover = std::min(QUAD_HANDOVER_PER_SM * sms, A.n); // the list holds n entries
         trace64_kernel<<<(unsigned)std::min(per_sm * sms, (work + 31) / 32), 32, 0, s>>>(A);
         const int rc = check_launch();

@@ -1,7 +1,8 @@
 """Double precision with four lanes per ray against one ray per lane.
 
-Queues of up to 200 rays per SM are traced by the four-lane kernel, longer ones
-by the one-lane kernel, whose last rays the four-lane kernel takes over.  Both
+Queues of up to 64 to 200 rays per SM (by step rule and order) are traced by
+the four-lane kernel, longer ones by the one-lane kernel, whose last rays the
+four-lane kernel takes over.  Both
 do the same operations on the same operands, so a ray's record is the same
 bits in each (no tolerance): an image alone, and as many copies of it in one
 buffer as pass the limit."""
