@@ -3200,8 +3200,10 @@ unsigned persistent_grid(const gray_ctx *ctx, const void *kernel, int block, int
 // fewer, most rays start at once in any order, and warps full of crawling rays
 // only crawl together (medians of 23 runs, three holes: 300^2 images 3.5 ms
 // ordered, 3.1 in natural order; 340^2 3.35 and 3.44; 370^2 3.48 and 3.60;
-// 400^2 3.61 and 3.77; 180000 mixed rays 4.7 and 5.3).  Nor under a step
-// budget that ends the pass too soon for its queue's order to matter.
+// 400^2 3.61 and 3.77; 180000 mixed rays 4.7 and 5.3; projections 420^2 1.14
+// and 1.29, 1024^2 4.15 and 4.82).  Not under Eq. 2, whose rays near a pole are
+// not the long ones (512^2: 3.4 ordered, 3.0 not), nor under a step budget that
+// ends the pass too soon for its queue's order to matter.
 constexpr int ORDER_MIN_BUDGET = 512;
 int64_t order_min_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512 * 8 / 5; }
 
@@ -3364,8 +3366,8 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             cudaEventRecord(ctx->ev[0], s);
             ctx->ev_used[0] = true;
         }
-        if (!order && ctx->opt.precision != GRAY_FP64 && !A.one_per_thread && n_state > order_min_rays(ctx) &&
-            (step_budget <= 0 || step_budget > ORDER_MIN_BUDGET)) {
+        if (!order && ctx->opt.precision != GRAY_FP64 && A.step_rule == GRAY_STEP_BENCH && !A.one_per_thread &&
+            n_state > order_min_rays(ctx) && (step_budget <= 0 || step_budget > ORDER_MIN_BUDGET)) {
             int *list = A.v.R ? A.v.R : A.v.L; // the zone pass fills R later; the other modes leave L unused
             order_rays_kernel<<<grid_for(n_state, ORDER_RAYS), ORDER_BLOCK, 0, s>>>(A.v, n_state, list, ctx->ws);
             if ((rc = check_launch()))

@@ -1,6 +1,6 @@
 """The lead-first queue of a trace without a caller's order.
 
-A trace of more than 1.6 times the rays that the single-precision pass holds at
+Under the benchmark rule a trace of more than 1.6 times the rays that the single-precision pass holds at
 once (512 per SM) orders its ACTIVE rays itself; a ray's result does not depend on its place in
 the queue, so every record equals, bit for bit (no tolerance), that of the
 same trace under an explicit order."""
@@ -52,7 +52,7 @@ def test_lead_first_queue_of_a_resumed_trace(image):
     side = int(math.isqrt(512 * 8 * sms // 5)) + 3
     im = I.Image(a=0.3, M=0.0, incl=1.0, nx=side, ny=side) if image == "flat" else \
         I.Image(a=0.9, incl=0.0, nx=side, ny=side)
-    opt = gray.Options(precision=gray.FP32_KAHAN_SEL64, max_steps=20000, r_sw=0.02, step_rule=gray.STEP_EQ2)
+    opt = gray.Options(precision=gray.FP32_KAHAN_SEL64, max_steps=20000, r_sw=0.02)
     got = trace(opt, im.n, lambda tr: tr.setup([im]), (513, 0), False)
     want = trace(opt, im.n, lambda tr: tr.setup([im]), (513, 0), True)
     assert got[1:] == want[1:] and got[1] == 0
