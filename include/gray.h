@@ -17,7 +17,9 @@
  *   - Units G = c = 1; lengths in units of M.  Angles in radians.
  *   - Buffers named *_dev are device pointers owned by the caller; buffers
  *     named *_host are host pointers owned by the caller.  The library owns
- *     only the gray_ctx and the small device workspace inside it.
+ *     only the gray_ctx, the small device workspace inside it and, once a
+ *     call passed more than eight images, a memory pool of the context's own
+ *     for its tables (given back by gray_destroy).
  *   - Every call that takes a stream enqueues its work on that stream
  *     (cudaStream_t passed as void*; NULL = legacy default stream) and
  *     returns without waiting, unless a host output pointer is given.
@@ -230,8 +232,9 @@ int gray_setup_rays(gray_ctx *ctx, const double *rays_dev, int64_t n, double M,
  * rays that entered the zone near the horizon (rays climbing out of it are
  * returned to a single-precision pass), then a last zone pass for the rays
  * that came back to the zone (in the zone's arithmetic there, in compensated
- * single precision once they leave it).  A ray's arithmetic does not depend
- * on which pass runs it.  Inside the single-precision pass, an Eq. 4 test
+ * single precision once they leave it).  In GRAY_FP64 short queues and the
+ * last rays of long ones are traced with four lanes per ray.  A ray's
+ * arithmetic does not depend on which pass or kernel runs it.  Inside the single-precision pass, an Eq. 4 test
  * whose outcome lies within single precision's rounding of its threshold
  * (near the ergosurface, where g_tt vanishes) is taken again in double-single
  * arithmetic.  With r_sw = 0.02 the final angles of every ray whose result
@@ -417,9 +420,9 @@ int gray_splat(gray_ctx *ctx, const void *state_dev, size_t state_bytes, int64_t
 /* gray_setup for callers that must not allocate device memory -- for
  * example a simulation code that owns the whole device memory budget through
  * its own pool, or a caller whose allocator calls are forbidden in its
- * time-critical loop.  gray_setup uploads the image table through a
- * temporary stream-ordered allocation on every call and needs a context,
- * whose creation allocates; this entry point needs neither.  The paper has no
+ * time-critical loop.  gray_setup uploads lists of more than eight images
+ * through a temporary stream-ordered allocation and needs a context, whose
+ * creation allocates; this entry point needs neither.  The paper has no
  * counterpart: it is an interface convenience of this library.
  *
  * It writes the same initial states as gray_setup (bit for bit) for a

@@ -7,6 +7,8 @@
 //   trace64_quad_kernel                      double precision with four lanes per ray
 //   zone_kernel<RETURN, T>                   the near-horizon zone of the
 //                                            selective mode (double-single or double)
+//   order_rays_kernel                        the queue of a large trace without an order
+//   begin_call_kernel, count_active_kernel   a call's counters, before and after its passes
 //   probe_rays_kernel, plan_*_kernel         the longest-first planner
 //   render_*, shadow_*, ring_*, splat        read-out of results
 //   eval_kernel<T>                           unit evaluations for parity tests
@@ -621,7 +623,8 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
 // so a zone step must never hold a warp of single-precision lanes; the
 // hand-off keeps the two populations apart and the single-precision kernel
 // free of the zone's registers.  GRAY_FP64 runs trace64_kernel over every
-// ray, with double planes.
+// ray, with double planes; its short queues and last rays go to
+// trace64_quad_kernel.
 
 enum : int { FLAG_DOUBLE_MODE = 1, FLAG_DOUBLE_REPR = 2 };
 
@@ -1233,7 +1236,7 @@ struct TeamShared {
 // Zone kernel of GRAY_FP32_KAHAN_SEL64: the rays of the hand-off list, in
 // extended precision T (double, or double-single on the single-precision
 // pipe: GRAY_ZONE_DS) while r < r_demote (= r_promote + r_sw).  RETURN = true
-// (first zone pass): double only; a ray that climbs out is stored as a
+// (first zone pass): extended precision only; a ray that climbs out is stored as a
 // compensated single pair and appended to the return list R, which the next
 // single-precision pass drains at full occupancy (this kernel holds no
 // single-precision state and fits three blocks per SM).  RETURN = false (last
@@ -1243,9 +1246,10 @@ struct TeamShared {
 // (T to hi, lo; exact for double-single), the same in both forms, so a ray's
 // arithmetic does not depend on which pass runs it.
 //
-// TEAM (double-single, first pass): once the list is drained and no more rays
-// are left in the block than a team holds, the warps list them in `sh` and
-// return, for zone_team to finish.
+// TEAM (double-single, first pass): ZONE_TAIL steps after the list is drained
+// and when no more rays are left in the block than a team holds, the warps
+// list them in `sh` and return, for zone_team to finish.  A warp's count only
+// falls once it is published, so the listed rays are at most 32.
 template <bool RETURN, typename T, int CFG, bool TEAM>
 __device__ __forceinline__ void zone_lanes(const TraceArgs &A, TeamShared *sh)
 {
