@@ -18,8 +18,9 @@
  *   - Buffers named *_dev are device pointers owned by the caller; buffers
  *     named *_host are host pointers owned by the caller.  The library owns
  *     only the gray_ctx, the small device workspace inside it and, once a
- *     call passed more than eight images, a memory pool of the context's own
- *     for its tables (given back by gray_destroy).
+ *     call needed a temporary table (more than eight images, ranges, rings),
+ *     a memory pool of the context's own that keeps at most 64 MB between
+ *     synchronisations (given back by gray_destroy).
  *   - Every call that takes a stream enqueues its work on that stream
  *     (cudaStream_t passed as void*; NULL = legacy default stream) and
  *     returns without waiting, unless a host output pointer is given.

@@ -236,7 +236,7 @@ struct gray_ctx {
     cudaStream_t side = nullptr;       // gray_setup_plan: the planning passes (high priority)
     cudaEvent_t fork = nullptr, join = nullptr;
     cudaStream_t cancel_stream = nullptr; // gray_cancel writes the flag through it (non-blocking)
-    cudaMemPool_t pool = nullptr;      // small temporary tables; keeps its memory until gray_destroy
+    cudaMemPool_t pool = nullptr;      // temporary tables (pool_alloc); destroyed by gray_destroy
 };
 
 namespace {
@@ -2937,10 +2937,12 @@ std::vector<ImageDev> image_table(const gray_image *images, int n_images, int64_
     return t;
 }
 
-// A temporary buffer on `stream` from the context's own pool, which keeps its
-// memory between calls (the device's default pool gives it back at every
-// synchronisation).  Freed with cudaFreeAsync.  Under stream capture the
+// A temporary buffer on `stream` from the context's own pool, which keeps up to
+// POOL_KEEP bytes between calls (the device's default pool gives all of it back
+// at every synchronisation; 64 MB hold the tables of 300 images many times
+// over, and a larger one-time scratch is given back).  Freed with cudaFreeAsync.  Under stream capture the
 // default pool serves, as a pool cannot be created there.
+constexpr uint64_t POOL_KEEP = 64ull << 20;
 int pool_alloc(gray_ctx *ctx, void **dev, size_t bytes, cudaStream_t s)
 {
     *dev = nullptr;
@@ -2954,8 +2956,13 @@ int pool_alloc(gray_ctx *ctx, void **dev, size_t bytes, cudaStream_t s)
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = ctx->device;
-        uint64_t keep = UINT64_MAX;
-        if (cudaMemPoolCreate(&ctx->pool, &props) != cudaSuccess)
+        uint64_t keep = POOL_KEEP;
+        // another stream of this thread may be under capture, which the call does not touch
+        cudaStreamCaptureMode mode = cudaStreamCaptureModeRelaxed;
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess)
+            return GRAY_ECUDA;
+        const cudaError_t made = cudaMemPoolCreate(&ctx->pool, &props);
+        if (cudaThreadExchangeStreamCaptureMode(&mode) != cudaSuccess || made != cudaSuccess)
             return GRAY_ECUDA;
         if (cudaMemPoolSetAttribute(ctx->pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess)
             return GRAY_ECUDA;
@@ -3211,7 +3218,6 @@ unsigned persistent_grid(const gray_ctx *ctx, const void *kernel, int block, int
 constexpr int ORDER_MIN_BUDGET = 512;
 int64_t order_min_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512 * 8 / 5; }
 
-// One single- or double-precision pass over the queue of A (no zone kernel).
 // A persistent single-precision pass.  A queue of up to three blocks per SM
 // (any small image) and the planner's probe pass take the instantiation without
 // the 128-register cap, three blocks of 128 threads to an SM: nothing is
@@ -3305,6 +3311,7 @@ int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
     return check_launch();
 }
 
+// One single- or double-precision pass over the queue of A (no zone kernel).
 int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s, Pass pass = Pass::Main)
 {
     if (A.one_per_thread && ctx->opt.precision != GRAY_FP64) {
