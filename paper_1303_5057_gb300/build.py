@@ -11,7 +11,7 @@ PKG = os.path.dirname(os.path.abspath(__file__))
 ROOT = os.path.dirname(PKG)
 SRC = os.path.join(PKG, "csrc", "gray.cu")
 DEPS = [SRC, os.path.join(PKG, "csrc", "kerr.cuh"), os.path.join(PKG, "csrc", "quad.cuh"),
-        os.path.join(ROOT, "include", "gray.h")]
+        os.path.join(PKG, "csrc", "tile.h"), os.path.join(ROOT, "include", "gray.h")]
 LIB = os.path.join(PKG, "libgray.so")
 ARCH = "-gencode=arch=compute_103a,code=sm_103a"
 

@@ -28,6 +28,7 @@
 #include "gray.h"
 #include "kerr.cuh"
 #include "quad.cuh"
+#include "tile.h"
 
 #include <cuda_runtime.h>
 
@@ -2057,13 +2058,9 @@ __global__ void plan_scatter_kernel(const __grid_constant__ ImageTable T, int n_
     int b = -1, ray = 0;
     if (valid) {
         const ImageDev &im = imgs[image_of(imgs, n_images, i)];
-        const unsigned p = (unsigned)(i - im.first), nx = (unsigned)im.nx;
-        const unsigned high = im.grid == GRAY_GRID_POLAR ? 1u : 4u; // rows of a strip
-        const unsigned strip = p / (high * nx), q = p - strip * high * nx;
-        const unsigned rows = min(high, (unsigned)im.ny - high * strip);
-        const unsigned col = rows == 4 ? q >> 2 : q / rows, row = high * strip + (q - col * rows);
-        b = plan_bucket(im, row, col, first_ray, stride, budget, S0);
-        ray = (int)(first_ray + im.first + (int64_t)row * nx + col);
+        const Pixel px = tile_pixel((unsigned)(i - im.first), (unsigned)im.nx, (unsigned)im.ny, im.grid == GRAY_GRID_POLAR);
+        b = plan_bucket(im, px.row, px.col, first_ray, stride, budget, S0);
+        ray = (int)(first_ray + im.first + (int64_t)px.row * im.nx + px.col);
     }
     const int lane = threadIdx.x & 31;
     const unsigned peers = __match_any_sync(FULL, b);
