@@ -3187,20 +3187,26 @@ TraceArgs make_trace_args(gray_ctx *ctx, void *state, int64_t n_state, int64_t s
     return A;
 }
 
-// Persistent grid: resident blocks per SM x SMs, never more blocks than work.
+// Blocks of a kernel that an SM holds at once, 0 if it holds none (its registers
+// at this block size exceed the register file).
+int resident_blocks(const void *kernel, int block)
+{
+    int per_sm = 0;
+    return cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) == cudaSuccess ? per_sm : 0;
+}
+
+// Persistent grid: `per_sm` blocks on each SM (the caller's option first),
+// never more blocks than work.
+unsigned persistent_grid(const gray_ctx *ctx, int per_sm, int block, int64_t work)
+{
+    if (ctx->opt.blocks_per_sm > 0)
+        per_sm = ctx->opt.blocks_per_sm;
+    const int64_t want = (int64_t)std::max(per_sm, 1) * ctx->num_sms, need = (work + block - 1) / block;
+    return (unsigned)std::max<int64_t>(std::min(want, need), 1);
+}
 unsigned persistent_grid(const gray_ctx *ctx, const void *kernel, int block, int64_t work)
 {
-    int per_sm = ctx->opt.blocks_per_sm;
-    if (per_sm <= 0) {
-        per_sm = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, 0) != cudaSuccess || per_sm < 1)
-            per_sm = 1;
-    }
-    int64_t want = (int64_t)per_sm * ctx->num_sms;
-    const int64_t need = (work + block - 1) / block;
-    if (want > need)
-        want = need;
-    return (unsigned)(want > 0 ? want : 1);
+    return persistent_grid(ctx, ctx->opt.blocks_per_sm > 0 ? 0 : resident_blocks(kernel, block), block, work);
 }
 
 // A trace without an order makes a lead-first queue of more than 1.6 times the
@@ -3220,7 +3226,11 @@ int64_t order_min_rays(const gray_ctx *ctx) { return (int64_t)ctx->num_sms * 512
 // the 128-register cap, three blocks of 128 threads to an SM: nothing is
 // re-formed under register pressure (probe pass 0.56 -> 0.52 ms, 32^2 image
 // 1.545 -> 1.519, 128^2 projection 0.431 -> 0.423); a longer one needs the
-// fourth block (1024^2: 7.98 ms capped, 8.5 uncapped).
+// fourth block (1024^2: 7.98 ms capped, 8.5 uncapped).  Of 256 or 384 threads
+// an SM holds one such block, and three blocks' rays are still faster in it
+// (256 threads, 250^2: 2.52 ms, 2.83 capped; 330^2: 2.89, 3.30).  Of more than
+// 448 it holds none (137 - 142 registers in the compensated modes): there the
+// capped instantiation, which fits up to 512, takes every queue.
 //
 // A probe pass beside the set-up of the other rays (gray_setup_plan) must
 // leave it room: three uncapped blocks take the whole register file, and the
@@ -3238,8 +3248,11 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
     const bool beside = pass == Pass::ProbeBesideSetup && work > BESIDE_BLOCKS_PER_SM * block * sms;
     if (!beside && (pass != Pass::Main || work <= SMALL_BLOCKS_PER_SM * block * sms)) {
         const auto kernel = trace32_kernel<MODE, 168, CFG>;
-        kernel<<<persistent_grid(ctx, (const void *)kernel, block, work), block, 0, s>>>(A);
-        return;
+        const int resident = resident_blocks((const void *)kernel, block);
+        if (resident > 0) {
+            kernel<<<persistent_grid(ctx, resident, block, work), block, 0, s>>>(A);
+            return;
+        }
     }
     const auto kernel = trace32_kernel<MODE, 128, CFG>;
     const unsigned grid = persistent_grid(ctx, (const void *)kernel, block, work);

@@ -440,6 +440,31 @@ def test_launch_shape_does_not_change_results(prec, shape):
     assert np.array_equal(got, ref)
 
 
+@pytest.mark.parametrize("options", [{}, {"stop_equator": 1}], ids=["", "equator"])
+@pytest.mark.parametrize("prec", [gray.FP32, gray.FP32_KAHAN, gray.FP32_KAHAN_SEL64])
+def test_blocks_up_to_512_threads(prec, options):
+    """Every block size whose registers fit an SM traces and plans queues of any
+    length, from one ray to a queue beyond the short ones' limit, with the bits
+    of the default size (results do not depend on the launch, so no tolerance)."""
+    small, large = I.Image(a=0.9, incl=1.2, nx=37, ny=29), I.Image(a=0.9, incl=1.2, nx=500, ny=500)
+    one = I.Image(a=0.9, incl=1.2, nx=1, ny=1, alpha0=3.0, alpha1=4.0, beta0=1.0, beta1=2.0)
+
+    def records(im, block, plan):
+        opt = gray.Options(precision=prec, max_steps=300, r_sw=0.02, block=block, **options)
+        tr = gray.Tracer(opt, im.n)
+        order = tr.setup_plan([im], probe_stride=4, probe_budget=50) if plan else tr.setup([im])
+        tr.trace(order=order if plan else None)
+        rec = tr.records()
+        tr.close()
+        return rec
+
+    for im, blocks in ((one, (512,)), (small, (32, 256, 384, 448, 480, 512)), (large, (256, 512))):
+        want = records(im, 0, False)
+        for block in blocks:
+            for plan in (False, True):
+                assert np.array_equal(records(im, block, plan), want, equal_nan=True), (im.n, block, plan)
+
+
 @pytest.mark.parametrize("prec", [gray.FP32_KAHAN_SEL64, gray.FP64])
 def test_setup_plan_equals_setup_then_plan(prec):
     """The fused call (non-probe set-up on a side stream, overlapping the
