@@ -92,6 +92,10 @@ extern "C" {
                                 /* size of its terms as the single-precision test evaluates them, the */
                                 /* test's ambiguity flag (1/0), its decision (1: redo), and the       */
                                 /* decision after the double-single re-test; 6 values                */
+#define GRAY_EVAL_XI_ZONE 8     /* in (M, a, eps_xi, y[8]) -> out, for y as double-single pairs        */
+                                /* (GRAY_FP32 only): the Eq. 4 decision of the zone's single-precision */
+                                /* test (1: redo), whether that test is certain of it (1/0), and the   */
+                                /* decision of the double-single test; 3 values                        */
 
 /* ---- launch of the trace kernel ------------------------------------- */
 #define GRAY_LAUNCH_PERSISTENT 0     /* persistent warps refilled from a work queue (default) */

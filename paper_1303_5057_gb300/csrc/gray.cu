@@ -2738,6 +2738,24 @@ __global__ void eval_kernel(int what, const double *in, int64_t n, double *out)
             out[6 * i + 4] = redo ? 1.0 : 0.0;
             out[6 * i + 5] = xi_fails_ds(y1, c1, aM, eps) ? 1.0 : 0.0;
         }
+    } else if (what == GRAY_EVAL_XI_ZONE) {
+        if constexpr (sizeof(T) == 4) {
+            const double *q = in + 11 * i;
+            const double M = q[0], a = q[1];
+            float c8[8];
+            hole_constants_f(a, M, 1000.0, c8);
+            const float2 low = make_float2((float)(a - (double)c8[0]), (float)(M - (double)c8[1]));
+            const Hole<ds> H = make_hole_ds(make_float4(c8[0], c8[1], c8[2], c8[3]),
+                                            make_float4(c8[4], c8[5], c8[6], c8[7]), low, ds(1.0), ds(1.0), ds(0.0));
+            ds y[8];
+            for (int m = 0; m < 8; ++m)
+                y[m] = ds(q[3 + m]);
+            const Geo<ds> g = geometry(H, y[1], y[2]);
+            bool certain;
+            out[3 * i] = xi_fails_high(H, g, y, ds(q[2]), certain) ? 1.0 : 0.0;
+            out[3 * i + 1] = certain ? 1.0 : 0.0;
+            out[3 * i + 2] = xi_fails<ds>(H, g, y, ds(q[2])) ? 1.0 : 0.0;
+        }
     } else if (what == GRAY_EVAL_XI) {
         const double *q = in + 10 * i;
         const Hole<T> H = cast_hole<T>(make_hole(q[1], q[0], 1.0, 1.0, 1.0, 0.0));
@@ -3944,7 +3962,7 @@ int gray_splat(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_s
 
 int gray_eval(int32_t what, int32_t precision, const double *in, int64_t n, double *out, void *stream)
 {
-    if (what < GRAY_EVAL_CHRISTOFFEL || what > GRAY_EVAL_NORM || n < 0)
+    if (what < GRAY_EVAL_CHRISTOFFEL || what > GRAY_EVAL_XI_ZONE || n < 0)
         return GRAY_EINVAL;
     if (precision != GRAY_FP64 && precision != GRAY_FP32)
         return GRAY_EINVAL;
