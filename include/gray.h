@@ -96,6 +96,9 @@ extern "C" {
                                 /* (GRAY_FP32 only): the Eq. 4 decision of the zone's single-precision */
                                 /* test (1: redo), whether that test is certain of it (1/0), and the   */
                                 /* decision of the double-single test; 3 values                        */
+#define GRAY_EVAL_FMA_DS 9      /* in (x, y, z) -> out, for their double-single pairs (GRAY_FP32 only): */
+                                /* both words of x y + z as the zone forms it, and of a normalised     */
+                                /* product and a sum; 4 values                                         */
 
 /* ---- launch of the trace kernel ------------------------------------- */
 #define GRAY_LAUNCH_PERSISTENT 0     /* persistent warps refilled from a work queue (default) */

@@ -2756,6 +2756,15 @@ __global__ void eval_kernel(int what, const double *in, int64_t n, double *out)
             out[3 * i + 1] = certain ? 1.0 : 0.0;
             out[3 * i + 2] = xi_fails<ds>(H, g, y, ds(q[2])) ? 1.0 : 0.0;
         }
+    } else if (what == GRAY_EVAL_FMA_DS) {
+        if constexpr (sizeof(T) == 4) {
+            const ds x(in[3 * i]), y(in[3 * i + 1]), z(in[3 * i + 2]);
+            const ds f = fma(x, y, z), p = ds_add(ds_mul(x, y), z);
+            out[4 * i] = (double)f.hi;
+            out[4 * i + 1] = (double)f.lo;
+            out[4 * i + 2] = (double)p.hi;
+            out[4 * i + 3] = (double)p.lo;
+        }
     } else if (what == GRAY_EVAL_XI) {
         const double *q = in + 10 * i;
         const Hole<T> H = cast_hole<T>(make_hole(q[1], q[0], 1.0, 1.0, 1.0, 0.0));
@@ -3962,7 +3971,7 @@ int gray_splat(gray_ctx *ctx, const void *state, size_t state_bytes, int64_t n_s
 
 int gray_eval(int32_t what, int32_t precision, const double *in, int64_t n, double *out, void *stream)
 {
-    if (what < GRAY_EVAL_CHRISTOFFEL || what > GRAY_EVAL_XI_ZONE || n < 0)
+    if (what < GRAY_EVAL_CHRISTOFFEL || what > GRAY_EVAL_FMA_DS || n < 0)
         return GRAY_EINVAL;
     if (precision != GRAY_FP64 && precision != GRAY_FP32)
         return GRAY_EINVAL;

@@ -26,7 +26,7 @@ FP64, FP32, FP32_KAHAN, FP32_KAHAN_SEL64 = 0, 1, 2, 3
 STEP_BENCH, STEP_EQ2 = 0, 1
 RENDER_PIXELS64, RENDER_PIXELS32, RENDER_RECORD, RENDER_INVARIANTS = 0, 1, 3, 4
 EVAL_CHRISTOFFEL, EVAL_RHS, EVAL_INITIAL, EVAL_XI, EVAL_SINCOS, EVAL_RECIP = 0, 1, 2, 3, 4, 5
-EVAL_SINCOS_DS, EVAL_NORM, EVAL_XI_ZONE = 6, 7, 8
+EVAL_SINCOS_DS, EVAL_NORM, EVAL_XI_ZONE, EVAL_FMA_DS = 6, 7, 8, 9
 LAUNCH_PERSISTENT, LAUNCH_ONE_PER_THREAD = 0, 1
 ZONE_DS, ZONE_FP64 = 0, 1
 GRID_CARTESIAN, GRID_POLAR = 0, 1
@@ -448,9 +448,9 @@ def gray_eval(what, precision, inp, stream=None):
     Returns a float64 CUDA tensor of n rows (see GRAY_EVAL_* in include/gray.h)."""
     import torch
     width_in = {EVAL_CHRISTOFFEL: 4, EVAL_RHS: 10, EVAL_INITIAL: 6, EVAL_XI: 10, EVAL_SINCOS: 1, EVAL_RECIP: 1,
-                EVAL_SINCOS_DS: 1, EVAL_NORM: 10, EVAL_XI_ZONE: 11}[what]
+                EVAL_SINCOS_DS: 1, EVAL_NORM: 10, EVAL_XI_ZONE: 11, EVAL_FMA_DS: 3}[what]
     width_out = {EVAL_CHRISTOFFEL: 64, EVAL_RHS: 8, EVAL_INITIAL: 8, EVAL_XI: 1, EVAL_SINCOS: 2, EVAL_RECIP: 2,
-                 EVAL_SINCOS_DS: 2, EVAL_NORM: 6, EVAL_XI_ZONE: 3}[what]
+                 EVAL_SINCOS_DS: 2, EVAL_NORM: 6, EVAL_XI_ZONE: 3, EVAL_FMA_DS: 4}[what]
     inp = inp.contiguous()
     n = inp.numel() // width_in
     out = torch.empty((n, width_out), dtype=torch.float64, device=inp.device)
