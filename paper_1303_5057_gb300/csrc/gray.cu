@@ -2194,7 +2194,9 @@ __global__ void __launch_bounds__(RECORD_BLOCK) render_record_kernel(StateView v
 }
 
 // GRAY_RENDER_INVARIANTS, in double from the stored state (bound by the FP64
-// pipe: a sine and cosine, a square root and three reciprocals per ray).
+// pipe: a sine and cosine, a square root and three divides per ray).  Reciprocals
+// in place of the divides rounded twice for their once, and gave NaN for a sin^2
+// below the normal range.
 __global__ void render_invariants_kernel(StateView v, int prec, int64_t first, int64_t n, double *out)
 {
     const int64_t j = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -2207,18 +2209,13 @@ __global__ void render_invariants_kernel(StateView v, int prec, int64_t first, i
     const Hole<double> H = make_hole(p.x, p.y, p.z, 1.0, 1.0, 0.0);
     double s, c;
     sincos(y[2], &s, &c);
-    // the metric of metric_pieces, with refined reciprocals for its divides
-    const double r = y[1], a2 = H.a * H.a, s2 = s * s;
-    const double Sigma = fma(a2, c * c, r * r), iS = recip(Sigma);
-    const double u = 2.0 * H.M * r * iS;
-    const double gtt = u - 1.0, gtp = -u * H.a * s2, gpp = (fma(r, r, a2) + u * a2 * s2) * s2;
-    const double grr = Sigma * recip(fma(r - H.rp, r - H.rm, H.dc));
+    const MetricPieces<double> m = metric_pieces(H, y[1], s, c);
     const double kt = y[4], kr = y[5], kh = y[6], kp = y[7];
-    const double E = -(gtt * kt + gtp * kp);
-    const double L = gtp * kt + gpp * kp;
-    const double kth_low = Sigma * kh;
-    const double Q = kth_low * kth_low + c * c * (-H.a * H.a * E * E + L * L * recip(s2));
-    const double N = gtt * kt * kt + 2.0 * gtp * kt * kp + grr * kr * kr + Sigma * kh * kh + gpp * kp * kp;
+    const double E = -(m.gtt * kt + m.gtp * kp);
+    const double L = m.gtp * kt + m.gpp * kp;
+    const double kth_low = m.gthth * kh;
+    const double Q = kth_low * kth_low + c * c * (-H.a * H.a * E * E + L * L / (s * s));
+    const double N = m.gtt * kt * kt + 2.0 * m.gtp * kt * kp + m.grr * kr * kr + m.gthth * kh * kh + m.gpp * kp * kp;
     double *o = out + 4 * j;
     o[0] = E;
     o[1] = L;
