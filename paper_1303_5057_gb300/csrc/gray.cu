@@ -374,9 +374,11 @@ __global__ void setup_rays_kernel(const double *rays, int64_t n, double M, int64
     double y[8];
     initial_state(M, q[2], q[4], q[3], q[0], q[1], y);
     float a_hi, a_lo, M_hi, M_lo;
-    split_pair(q[2], a_hi, a_lo); // the low word of a is a - a_hi, of opposite sign
+    // the low word of a is a - a_hi, of opposite sign (0 - x: a zero stays +0)
+    split_pair(q[2], a_hi, a_lo);
     split_pair(M, M_hi, M_lo);
-    store_initial(v, prec, first_ray + i, y, q[2], M, q[4], nullptr, make_float2(-a_lo, -M_lo));
+    store_initial(v, prec, first_ray + i, y, q[2], M, q[4], nullptr,
+                  make_float2(0.0f - a_lo, 0.0f - M_lo));
 }
 
 // --------------------------------------------------------------------------

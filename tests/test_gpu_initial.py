@@ -37,3 +37,21 @@ def test_initial_pairs_are_the_rounded_doubles(precision, r_obs):
     assert np.array_equal(got[:, 8:16], hi.astype(np.float64) - lo.astype(np.float64))
     assert np.array_equal(got[:, 4:8], hi[:, :4].astype(np.float64))
     assert np.all(got[:, :4] == 0) and np.all(got[:, 16] == 0)
+
+
+def test_single_rays_keep_the_constants_of_images_bit_for_bit():
+    """A ray set up by itself stores the same constants as a one-pixel image with
+    its hole: spin, mass, distance and the spin's and mass's low words (a zero
+    low word is +0)."""
+    spins = [0.0, 0.5, -0.5, 0.3, -0.3, 0.9, 0.998, 1e-9]
+    n = len(spins)
+    images = [I.Image(a=a, incl=1.0, nx=1, ny=1, alpha0=2.0, alpha1=4.0, beta0=1.0, beta1=3.0) for a in spins]
+    rays = torch.tensor([[3.0, 2.0, a, 1.0, images[0].r_obs] for a in spins], dtype=torch.float64, device="cuda")
+    plane = (32 * n + 255) // 256 * 256  # FP64: position, momentum, final point, constants
+    stored = []
+    for lone in (False, True):
+        tr = gray.Tracer(gray.Options(precision=gray.FP64), n)
+        tr.setup_rays(rays) if lone else tr.setup(images)
+        stored.append(tr.state[3 * plane:3 * plane + 32 * n].cpu().numpy())
+        tr.close()
+    assert np.array_equal(stored[0], stored[1])
