@@ -987,8 +987,13 @@ __global__ void __launch_bounds__(32) trace64_kernel(TraceArgs A)
             if ((int64_t)base + cnt >= nq)
                 exhausted = true;
         }
-        if (!__any_sync(FULL, has))
+        if (!__any_sync(FULL, has)) {
+            // slots passed over since the last report count for the others' hand-over
+            const unsigned r = A.handover > 0 ? __reduce_add_sync(FULL, resolved) : 0;
+            if (lane == 0 && r)
+                atomicAdd(&A.ws->demoted, (unsigned long long)r);
             break;
+        }
 
         if (give) {
             int rank;

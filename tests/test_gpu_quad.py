@@ -72,3 +72,28 @@ def test_a_short_state_with_a_long_queue_keeps_its_hand_off_list():
     rec = tr.records()
     tr.close()
     assert rc == 0 and n_active == 0 and np.array_equal(rec, want)
+
+
+def test_few_rays_of_a_long_buffer_reach_the_four_lane_kernel():
+    """Warps that pass over finished or empty slots only count them as well, so
+    the few rays left of a long buffer are handed over (the hand-off list is the
+    state's last plane) and end with the bits of a trace alone."""
+    im = I.Image(a=0.9, incl=1.0, nx=40, ny=30)
+    opt = gray.Options(precision=gray.FP64, max_steps=20000)
+    want = records([im], opt, (0,))
+    n = 300 * torch.cuda.get_device_properties(0).multi_processor_count
+    tr = gray.Tracer(opt, n)
+    gray.gray_clear(tr.ctx, tr.state, n, 0, n)
+    tr.setup([im], first_ray=n // 2)
+    plane = lambda size: (size * n + 255) // 256 * 256
+    first = 4 * plane(32) + 2 * plane(16)
+    listed = tr.state[first:first + 4 * n].view(torch.int32)
+    listed.fill_(-1)
+    _, n_active, _ = tr.trace()
+    rec = tr.records(first_ray=n // 2, n=im.n)
+    rays = listed.cpu().numpy()
+    rays = rays[rays >= 0]
+    tr.close()
+    assert n_active == 0 and np.array_equal(rec, want, equal_nan=True)
+    assert len(rays) > im.n // 2 and len(set(rays)) == len(rays)
+    assert rays.min() >= n // 2 and rays.max() < n // 2 + im.n
