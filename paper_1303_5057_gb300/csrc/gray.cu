@@ -387,20 +387,23 @@ __global__ void setup_rays_kernel(const double *rays, int64_t n, double M, int64
 // the final point on the stop surface -> Eq. 3 remap.
 // --------------------------------------------------------------------------
 
-// State update y1 = y + inc, plain or compensated (Kahan: the true value is
-// y - c).
+// State update y1 = y + h v, plain or compensated (Kahan: the true value is
+// y - c).  In double r, theta and the momentum take the product and the sum with
+// one rounding, t and phi with two (see plain_add).
 template <typename T, bool KAHAN>
-__device__ __forceinline__ void add_update(const T *y, const T *c, const T *inc, T *y1, T *c1)
+__device__ __forceinline__ void add_update(const T *y, const T *c, T h, const T *v, T *y1, T *c1)
 {
 #pragma unroll
     for (int m = 0; m < 8; ++m) {
         if (KAHAN) {
-            const T d = inc[m] - c[m];
+            const T d = h * v[m] - c[m];
             const T t = y[m] + d;
             c1[m] = (t - y[m]) - d;
             y1[m] = t;
+        } else if (m == 0 || m == 3) {
+            y1[m] = plain_add(y[m], h * v[m]);
         } else {
-            y1[m] = y[m] + inc[m];
+            y1[m] = mul_add(h, v[m], y[m]);
         }
     }
 }
@@ -458,8 +461,7 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
     accel_geo(H, g, y[4], y[5], y[6], y[7], a1);
     const T hh = scaled(h, 0.5);
     const T dr = KAHAN ? -c[1] : T(0), dth = KAHAN ? -c[2] : T(0);
-    const T h6 = sixth(h);
-    T inc[8];
+    T v[8]; // the sums k1 + 2 k2 + 2 k3 + k4 and likewise of the accelerations
     if constexpr (std::is_same<T, ds>::value) {
         // double-single (the zone): the three later stages in one rolled loop,
         // one copy of the stage's ~8x longer code (the zone pass is 1.6x
@@ -493,11 +495,11 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
         }
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            inc[m] = h6 * sk[m];
-            inc[4 + m] = h6 * sa[m];
+            v[m] = sk[m];
+            v[4 + m] = sa[m];
         }
     } else {
-        T a2[4], a3[4], a4[4];
+        T a2[4], a3[4];
         const T r2 = fma(hh, y[5], y[1]), th2 = fma(hh, y[6], y[2]);
         const T kt2 = fma(hh, a1[0], y[4]), kr2 = fma(hh, a1[1], y[5]), kh2 = fma(hh, a1[2], y[6]),
                 kp2 = fma(hh, a1[3], y[7]);
@@ -509,17 +511,18 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
         const T r4 = fma(h, kr3, y[1]), th4 = fma(h, kh3, y[2]);
         const T kt4 = fma(h, a3[0], y[4]), kr4 = fma(h, a3[1], y[5]), kh4 = fma(h, a3[2], y[6]),
                 kp4 = fma(h, a3[3], y[7]);
-        accel_geo(H, geometry_rel(H, g, r4, h * kh3, th4, dr, dth), kt4, kr4, kh4, kp4, a4);
-        inc[0] = h6 * (y[4] + T(2) * (kt2 + kt3) + kt4);
-        inc[1] = h6 * (y[5] + T(2) * (kr2 + kr3) + kr4);
-        inc[2] = h6 * (y[6] + T(2) * (kh2 + kh3) + kh4);
-        inc[3] = h6 * (y[7] + T(2) * (kp2 + kp3) + kp4);
+        T fa[4], fb[4];
+        accel_factors(H, geometry_rel(H, g, r4, h * kh3, th4, dr, dth), kt4, kr4, kh4, kp4, fa, fb);
+        v[0] = y[4] + T(2) * (kt2 + kt3) + kt4;
+        v[1] = y[5] + T(2) * (kr2 + kr3) + kr4;
+        v[2] = y[6] + T(2) * (kh2 + kh3) + kh4;
+        v[3] = y[7] + T(2) * (kp2 + kp3) + kp4;
 #pragma unroll
         for (int m = 0; m < 4; ++m)
-            inc[4 + m] = h6 * (a1[m] + T(2) * (a2[m] + a3[m]) + a4[m]);
+            v[4 + m] = mul_add(fa[m], fb[m], mul_add(T(2), plain_add(a2[m], a3[m]), a1[m]));
     }
     T y1[8], c1[8];
-    add_update<T, KAHAN>(y, c, inc, y1, c1);
+    add_update<T, KAHAN>(y, c, sixth(h), v, y1, c1);
     Geo<T> g1 = geometry(H, y1[1], y1[2], KAHAN ? -c1[1] : T(0), KAHAN ? -c1[2] : T(0));
 
     // Eq. 4 monitor: redo the step as forward Euler at h/9 when |xi + 1| > eps.
@@ -542,10 +545,10 @@ __device__ __forceinline__ int step_once(const Hole<T> &H, const StepOpt<T> &O, 
         h = ninth(h);
 #pragma unroll
         for (int m = 0; m < 4; ++m) {
-            inc[m] = h * y[4 + m];
-            inc[4 + m] = h * a1[m];
+            v[m] = y[4 + m];
+            v[4 + m] = a1[m];
         }
-        add_update<T, KAHAN>(y, c, inc, y1, c1);
+        add_update<T, KAHAN>(y, c, h, v, y1, c1);
         g1 = geometry(H, y1[1], y1[2], KAHAN ? -c1[1] : T(0), KAHAN ? -c1[2] : T(0));
         ++euler;
     }

@@ -115,7 +115,11 @@ __host__ __device__ inline Hole<double> make_hole(double a, double M, double r_o
     H.t2a = 2.0 * a;
     H.t2a2 = 2.0 * H.a2;
     H.t2Ma = 2.0 * H.Ma;
+#ifdef __CUDA_ARCH__
+    double disc = fma(M, M, -(a * a)); // the same in every kernel (see plain_add)
+#else
     double disc = M * M - a * a;
+#endif
     double root = disc > 0.0 ? sqrt(disc) : 0.0;
     H.rp = M + root;
     H.rm = M - root;
@@ -316,6 +320,16 @@ __device__ __forceinline__ double recip_approx(double x) { return recip(x); }
 template <typename T> __device__ __forceinline__ T scaled(T x, double k) { return T(k) * x; }
 template <typename T> __device__ __forceinline__ T fma_scaled(T x, double k, T c) { return fma(x, T(k), c); }
 
+// A sum that takes its terms as rounded, and a product-sum with one rounding.
+// Double is traced by two kernels that must agree bit for bit (one lane per ray,
+// and four in quad.cuh), so wherever a product meets a sum the step's source says
+// which of the two is meant and leaves the compiler's contraction no choice.
+// Single precision leaves it to the compiler; double-single has none.
+template <typename T> __device__ __forceinline__ T plain_add(T x, T y) { return x + y; }
+__device__ __forceinline__ double plain_add(double x, double y) { return __dadd_rn(x, y); }
+template <typename T> __device__ __forceinline__ T mul_add(T x, T y, T z) { return z + x * y; }
+__device__ __forceinline__ double mul_add(double x, double y, double z) { return ::fma(x, y, z); }
+
 // Geometry of one point (r, theta): the quantities every right-hand side and
 // the Eq. 4 monitor need, with the reciprocals of Sigma, Delta and sin(theta).
 template <typename T> struct Geo {
@@ -453,13 +467,16 @@ __device__ __forceinline__ Geo<T> geometry_rel(const Hole<T> &H, const Geo<T> &g
 //            - 2 r k^r k^th ] / Sigma
 //   a^ph = -2 [ u ((M a A X - 2 M r^2 k^ph)/Sigma + r k^ph)
 //               + cot(th) k^th (k^ph - Z/Sigma) ]
+//
+// Each component is the product of two factors, fa and fb: RK4's last stage takes
+// them into its sum of accelerations with one rounding.
 template <typename T>
-__device__ __forceinline__ void accel_geo(const Hole<T> &H, const Geo<T> &g, T kt, T kr, T kh, T kp, T *acc)
+__device__ __forceinline__ void accel_factors(const Hole<T> &H, const Geo<T> &g, T kt, T kr, T kh, T kp, T *fa, T *fb)
 {
     const T r = g.r, iS = g.iS;
     const T r2 = r * r, s2 = g.s * g.s, sc = g.s * g.c;
     const T A = fma_scaled(r2, 2.0, -g.Sigma);
-    const T P = r2 + H.a2;
+    const T P = plain_add(r2, H.a2);
     const T V = -(H.t2a * s2) * kp;
     const T X = fma_scaled(V, 0.5, kt) * iS;
     const T u = kr * g.iD;
@@ -468,21 +485,35 @@ __device__ __forceinline__ void accel_geo(const Hole<T> &H, const Geo<T> &g, T k
     // t
     const T ut = fma(P * A, X, r2 * V);
     const T xt = -(H.t2a2 * (r * sc)) * (kh * X);
-    acc[0] = (H.m2M * iS) * fma(u, ut, xt);
+    fa[0] = H.m2M * iS;
+    fb[0] = fma(u, ut, xt);
     // r
     const T DX = g.Delta * X;
     T sr = fma(H.M * A, fma(-DX, X, q), (g.Delta * r) * fma(s2, kp2, kh2));
     sr = fma(-((H.a2 * r) * s2), q, sr);
     sr = fma(H.t2a2 * sc, krkh, sr);
-    acc[1] = iS * sr;
+    fa[1] = iS;
+    fb[1] = sr;
     // theta
     const T Z = (H.t2Ma * r) * X;
-    const T hth = fma(Z, fma(H.a, X, scaled(kp, -2.0)), fma(P, kp2, H.a2 * (kh2 - q)));
-    acc[2] = iS * fma_scaled(r * krkh, -2.0, sc * hth);
+    const T hth = fma(Z, fma(H.a, X, scaled(kp, -2.0)), fma(P, kp2, H.a2 * plain_add(kh2, -q)));
+    fa[2] = iS;
+    fb[2] = fma_scaled(r * krkh, -2.0, sc * hth);
     // phi
     const T inner = fma(iS, fma(H.m2M * r2, kp, (H.Ma * A) * X), r * kp);
     const T up2 = fma(-Z, iS, kp);
-    acc[3] = scaled(fma(u, inner, ((g.c * g.is) * kh) * up2), -2.0);
+    fa[3] = T(-2.0);
+    fb[3] = fma(u, inner, ((g.c * g.is) * kh) * up2);
+}
+template <typename T>
+__device__ __forceinline__ void accel_geo(const Hole<T> &H, const Geo<T> &g, T kt, T kr, T kh, T kp, T *acc)
+{
+    T fa[4], fb[4];
+    accel_factors(H, g, kt, kr, kh, kp, fa, fb);
+    acc[0] = fa[0] * fb[0];
+    acc[1] = fa[1] * fb[1];
+    acc[2] = fa[2] * fb[2];
+    acc[3] = scaled(fb[3], -2.0);
 }
 
 // Eq. 4 test without its division: |xi + 1| > eps  <=>
@@ -787,7 +818,7 @@ template <typename T> __device__ __forceinline__ T step_size(const Hole<T> &H, c
     const T guard = (r - H.r_h) * scaled(recip(fabs(kr)), 0.5);
     T h;
     if (O.step_rule == 1)
-        h = fmin(O.h_frac * recip(fabs(kr) * recip(r) + fabs(y[6]) + fabs(y[7])), guard);
+        h = fmin(O.h_frac * recip(mul_add(fabs(kr), recip(r), fabs(y[6])) + fabs(y[7])), guard);
     else
         h = fmin(O.h_frac * r, guard);
     h = fmax(h, O.h_min);

@@ -17,8 +17,9 @@
 // the exchange latency between slots, not the pipe, is what is left.
 //
 // Every value is formed by the same operations on the same operands as in
-// step_once<double, false>, with every product-sum contraction written out,
-// so a ray's result is the same bits in both.  A product alone is taken as
+// step_once<double, false>, with every product-sum contraction written out on
+// both sides (plain_add, mul_add and fma there), so a ray's result is the same
+// bits in both whatever the compiler does.  A product alone is taken as
 // fma(x, y, -0), which rounds and signs as x * y does.
 //
 // All lanes of the warp run every slot (idle quads on a harmless state), so
@@ -252,16 +253,16 @@ __device__ __forceinline__ QuadStep quad_step(const Hole<double> &H, const StepO
             tk = ks;
             ta = as;
         } else if (stage == 1) {
-            tk += ks;
-            ta += as;
+            tk = plain_add(tk, ks);
+            ta = plain_add(ta, as);
         }
     }
     const double h6 = h * (1.0 / 6.0), h9 = h * (1.0 / 9.0);
     const bool tp = m == 0 || m == 3;
-    double x1 = fma(h6, fma(2.0, tk, k0) + ks, tp ? -0.0 : x0);
+    double x1 = fma(h6, plain_add(fma(2.0, tk, k0), ks), tp ? -0.0 : x0);
     double k1 = fma(h6, fma(fa, fb, fma(2.0, ta, a1)), k0);
     if (tp)
-        x1 += x0;
+        x1 = plain_add(x1, x0);
 
     // sin and cos of the new angle in lanes 0 and 1, and of the angle a
     // forward-Euler redo would end at in lanes 2 and 3: a ray that crawls on
@@ -287,7 +288,7 @@ __device__ __forceinline__ QuadStep quad_step(const Hole<double> &H, const StepO
                           qget(ke, 1), qget(ke, 2), qget(ke, 3), ge, qe);
         if (redo) {
             h = h9;
-            x1 = tp ? xe + x0 : xe;
+            x1 = tp ? plain_add(xe, x0) : xe;
             k1 = ke;
             g1 = ge;
             pre = qe;

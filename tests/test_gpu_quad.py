@@ -97,3 +97,24 @@ def test_few_rays_of_a_long_buffer_reach_the_four_lane_kernel():
     assert n_active == 0 and np.array_equal(rec, want, equal_nan=True)
     assert len(rays) > im.n // 2 and len(set(rays)) == len(rays)
     assert rays.min() >= n // 2 and rays.max() < n // 2 + im.n
+
+
+@pytest.mark.parametrize("name", CASES)
+def test_one_lane_kernel_alone_gives_the_bits_of_four(name):
+    """Fewer steps per call than lie between two refills (16): every ray yields
+    inside its first block of steps, before any can be handed over, so the whole
+    trajectory stays with the one-lane kernel, the longest rays' ends included."""
+    im, options = CASES[name]
+    opt = gray.Options(precision=gray.FP64, **{"max_steps": 20000, **options})
+    alone = records([im], opt, (0,))
+    limit = 200 * torch.cuda.get_device_properties(0).multi_processor_count
+    copies = limit // im.n + 1
+    tr = gray.Tracer(opt, copies * im.n)
+    tr.setup([im] * copies)
+    n_active = 1
+    while n_active:
+        _, n_active, _ = tr.trace(step_budget=15)
+    rec = tr.records().reshape(copies, im.n, -1)
+    tr.close()
+    same = (rec == alone[None]) | (np.isnan(rec) & np.isnan(alone[None]))
+    assert np.all(same), np.argwhere(~same)[:5]
