@@ -3323,26 +3323,34 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
 // and 15.3, but 120^2: 21.1 and 17.1, 158^2: 27.0 and 19.1).  In longer queues
 // the one-lane kernel hands its last rays over (A.handover; 300 x 211 natural
 // order 62 -> 51, Eq. 2 48 -> 44; 16 to 64 rays per SM are within 2 % of each
-// other).
+// other).  An order of the caller's counts as planned, whatever it is.
+//
+// Probe passes are the planner's budget of steps for every probe: no ray is much
+// longer than the others, and the four-lane kernel is the faster one only as far
+// as it holds them all at once, 48 per SM (plan of a 440^2 image, 36 probes per
+// SM: 5.3 ms, one-lane 9.0; 512^2, 49: 7.9 and 7.0; 1024^2, 192: 20.9 and 14.2).
+// Nor is there a last ray to hand over (800^2: 8.4 with, 7.8 without).
 constexpr int W64_PER_SM = 4, W64_PER_SM_LONG = 5, LONG_RAYS_PER_SM = 2048;
 constexpr int QUAD_PER_SM = 6, QUAD_HANDOVER_PER_SM = 32;
 constexpr int QUAD_RAYS_PLANNED = 200, QUAD_RAYS_ANY_ORDER = 80, QUAD_RAYS_EQ2 = 64; // per SM
+constexpr int QUAD_RAYS_PROBES = 8 * QUAD_PER_SM;
 
-int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, cudaStream_t s)
+int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, Pass pass, cudaStream_t s)
 {
     const int64_t sms = ctx->num_sms;
     int64_t per_sm = ctx->opt.blocks_per_sm > 0       ? 4 * (int64_t)ctx->opt.blocks_per_sm
                      : work > LONG_RAYS_PER_SM * sms ? W64_PER_SM_LONG
                                                      : W64_PER_SM;
     int64_t quad_work = work;
-    const int quad_rays = A.step_rule == GRAY_STEP_EQ2 ? QUAD_RAYS_EQ2
-                          : A.order                    ? QUAD_RAYS_PLANNED
-                                                       : QUAD_RAYS_ANY_ORDER;
+    const int quad_rays = pass != Pass::Main             ? QUAD_RAYS_PROBES
+                          : A.step_rule == GRAY_STEP_EQ2 ? QUAD_RAYS_EQ2
+                          : A.order                      ? QUAD_RAYS_PLANNED
+                                                         : QUAD_RAYS_ANY_ORDER;
     if (work > quad_rays * sms) {
-        A.handover = std::min(QUAD_HANDOVER_PER_SM * sms, A.n); // the list holds n entries
+        A.handover = pass == Pass::Main ? std::min(QUAD_HANDOVER_PER_SM * sms, A.n) : 0; // the list holds n entries
         trace64_kernel<<<(unsigned)std::min(per_sm * sms, (work + 31) / 32), 32, 0, s>>>(A);
         const int rc = check_launch();
-        if (rc)
+        if (rc || !A.handover)
             return rc;
         A.handover = 0;
         A.order = A.v.L;
@@ -3379,7 +3387,7 @@ int launch_pass(gray_ctx *ctx, const TraceArgs &A, int64_t work, cudaStream_t s,
     const int block = ctx->opt.block > 0 ? ctx->opt.block : 128;
     switch (ctx->opt.precision) {
     case GRAY_FP64:
-        return launch_trace64(ctx, A, work, s);
+        return launch_trace64(ctx, A, work, pass, s);
     case GRAY_FP32:
         launch_trace32<GRAY_FP32>(ctx, A, work, block, pass, s);
         break;

@@ -54,3 +54,22 @@ def test_planned_queue_is_a_permutation(name, fused):
     _, n_active, _ = tr.trace(order=torch.from_numpy(q).cuda())
     assert n_active == 0
     tr.close()
+
+
+@pytest.mark.parametrize("side", [80, 84, 88, 150])
+def test_double_precision_probes_advance_as_a_trace(side):
+    """Around 48 probes per SM the planner's probe pass changes kernel: with every
+    pixel a probe, its states are those of a trace of the same budget."""
+    im = I.Image(a=0.9, incl=1.2, nx=side, ny=side)
+    recs = []
+    for plan in (True, False):
+        tr = gray.Tracer(gray.Options(precision=gray.FP64, max_steps=20000), im.n)
+        if plan:
+            q = tr.setup_plan([im], probe_stride=1, probe_budget=40)
+            assert np.array_equal(np.sort(q.cpu().numpy()), np.arange(im.n))
+        else:
+            tr.setup([im])
+            tr.trace(step_budget=40)
+        recs.append(tr.records())
+        tr.close()
+    assert np.array_equal(recs[0], recs[1], equal_nan=True)
