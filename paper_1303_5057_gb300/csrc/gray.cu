@@ -3325,29 +3325,42 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
 // order 62 -> 51, Eq. 2 48 -> 44; 16 to 64 rays per SM are within 2 % of each
 // other).  An order of the caller's counts as planned, whatever it is.
 //
-// Probe passes are the planner's budget of steps for every probe: no ray is much
-// longer than the others, and the four-lane kernel is the faster one only as far
-// as it holds them all at once, 48 per SM (plan of a 440^2 image, 36 probes per
-// SM: 5.3 ms, one-lane 9.0; 512^2, 49: 7.9 and 7.0; 1024^2, 192: 20.9 and 14.2).
-// Nor is there a last ray to hand over (800^2: 8.4 with, 7.8 without).
+// Probe passes, and calls with a budget of up to 512 steps, are the same steps
+// for nearly every ray: no ray is much longer than the others, and the four-lane
+// kernel is the faster one only as far as it holds them all at once, 48 per SM
+// (plan of a 440^2 image, 36 probes per SM: 5.3 ms, one-lane 9.0; 512^2, 49: 7.9
+// and 7.0; 1024^2, 192: 20.9 and 14.2; 50 steps of 59 rays per SM 1.50 and 0.80).
+// Nor is there a last ray to hand over (plan of 800^2: 8.4 with, 7.8 without; 50
+// steps of 80 rays per SM 1.62 and 0.80).  With a budget that few rays end within
+// more warps hide each other's refills: eight per SM up to 256 steps (50 steps of
+// 129 rays per SM 1.66 -> 1.22 ms, of 1645 11.5 -> 11.2; 400 of 592 35.5 -> 38.0,
+// so no further).  Up to 32 steps do not pay the four-lane kernel's longer start
+// either (8 steps of 24 rays per SM 0.20 and 0.15 ms, 50 steps 0.72 and 0.80).
+// Budgets from 512 to 1024 keep the 48 and hand over (700 steps of 80 rays per SM:
+// 13.9 from the four-lane kernel, 11.5).
 constexpr int W64_PER_SM = 4, W64_PER_SM_LONG = 5, LONG_RAYS_PER_SM = 2048;
 constexpr int QUAD_PER_SM = 6, QUAD_HANDOVER_PER_SM = 32;
 constexpr int QUAD_RAYS_PLANNED = 200, QUAD_RAYS_ANY_ORDER = 80, QUAD_RAYS_EQ2 = 64; // per SM
-constexpr int QUAD_RAYS_PROBES = 8 * QUAD_PER_SM;
+constexpr int QUAD_RAYS_EVEN = 8 * QUAD_PER_SM;
+constexpr int TINY_BUDGET = 32, SHORT_BUDGET = 256, EVEN_BUDGET = 512, W64_PER_SM_SHORT = 8;
 
 int launch_trace64(gray_ctx *ctx, TraceArgs A, int64_t work, Pass pass, cudaStream_t s)
 {
     const int64_t sms = ctx->num_sms;
-    int64_t per_sm = ctx->opt.blocks_per_sm > 0       ? 4 * (int64_t)ctx->opt.blocks_per_sm
+    const int64_t budget = A.budget > 0 ? A.budget : INT64_MAX;
+    const bool even = pass != Pass::Main || budget <= EVEN_BUDGET; // the same steps for nearly every ray
+    int64_t per_sm = ctx->opt.blocks_per_sm > 0      ? 4 * (int64_t)ctx->opt.blocks_per_sm
+                     : budget <= SHORT_BUDGET        ? W64_PER_SM_SHORT
                      : work > LONG_RAYS_PER_SM * sms ? W64_PER_SM_LONG
                                                      : W64_PER_SM;
     int64_t quad_work = work;
-    const int quad_rays = pass != Pass::Main             ? QUAD_RAYS_PROBES
-                          : A.step_rule == GRAY_STEP_EQ2 ? QUAD_RAYS_EQ2
-                          : A.order                      ? QUAD_RAYS_PLANNED
-                                                         : QUAD_RAYS_ANY_ORDER;
+    const int quad_rays = budget <= TINY_BUDGET                   ? 0
+                          : even || budget <= 2 * EVEN_BUDGET     ? QUAD_RAYS_EVEN
+                          : A.step_rule == GRAY_STEP_EQ2          ? QUAD_RAYS_EQ2
+                          : A.order                               ? QUAD_RAYS_PLANNED
+                                                                  : QUAD_RAYS_ANY_ORDER;
     if (work > quad_rays * sms) {
-        A.handover = pass == Pass::Main ? std::min(QUAD_HANDOVER_PER_SM * sms, A.n) : 0; // the list holds n entries
+        A.handover = even ? 0 : std::min(QUAD_HANDOVER_PER_SM * sms, A.n); // the list holds n entries
         trace64_kernel<<<(unsigned)std::min(per_sm * sms, (work + 31) / 32), 32, 0, s>>>(A);
         const int rc = check_launch();
         if (rc || !A.handover)

@@ -118,3 +118,14 @@ def test_one_lane_kernel_alone_gives_the_bits_of_four(name):
     tr.close()
     same = (rec == alone[None]) | (np.isnan(rec) & np.isnan(alone[None]))
     assert np.all(same), np.argwhere(~same)[:5]
+
+
+@pytest.mark.parametrize("side", [84, 88, 150])
+def test_budgets_do_not_change_results(side):
+    """Calls of few steps, of some and of all take different kernels and
+    hand-overs around 48 rays per SM; a ray's record is the same bits."""
+    im = I.Image(a=0.95, incl=math.radians(80.0), nx=side, ny=side)
+    opt = gray.Options(precision=gray.FP64, max_steps=20000)
+    want = records([im], opt, (0,))
+    for budgets in ((40, 600, 0), (512, 512, 0), (1024, 1025, 0), (1,) * 5 + (0,)):
+        assert np.array_equal(records([im], opt, budgets), want, equal_nan=True), budgets
