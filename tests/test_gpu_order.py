@@ -57,3 +57,22 @@ def test_lead_first_queue_of_a_resumed_trace(image):
     want = trace(opt, im.n, lambda tr: tr.setup([im]), (513, 0), True)
     assert got[1:] == want[1:] and got[1] == 0
     assert np.array_equal(got[0], want[0], equal_nan=True)
+
+
+@pytest.mark.parametrize("surplus", [-1, 0, 1])
+def test_as_many_active_rays_as_the_limit(surplus):
+    """The limit counts ACTIVE rays: below and at it the pass takes the buffer as
+    it lies, above it the lead-first queue."""
+    limit = 512 * 8 * torch.cuda.get_device_properties(0).multi_processor_count // 5
+    n = limit + 4000
+    opt = gray.Options(precision=gray.FP32_KAHAN_SEL64, max_steps=20000, r_sw=0.02)
+    rays = torch.from_numpy(I.mixed_rays(n, offset=5 * n)).cuda()
+
+    def prepare(tr):
+        tr.setup_rays(rays)
+        gray.gray_clear(tr.ctx, tr.state, n, 501, 4000 - surplus)
+
+    got = trace(opt, n, prepare, (0,), False)
+    want = trace(opt, n, prepare, (0,), True)
+    assert got[1:] == want[1:] and got[1] == 0
+    assert np.array_equal(got[0], want[0], equal_nan=True)
