@@ -955,13 +955,17 @@ __global__ void __launch_bounds__(32) trace64_kernel(TraceArgs A)
         if (A.handover > 0 && !stop) {
             const unsigned r = __reduce_add_sync(FULL, resolved);
             resolved = 0;
-            long long left = 0;
+            bool few = false;
             if (lane == 0) {
                 if (r)
                     atomicAdd(&A.ws->demoted, (unsigned long long)r);
-                left = nq - (long long)*(volatile unsigned long long *)&A.ws->demoted;
+                // the queue's head, not this warp's own refills, tells that the queue is
+                // empty: a warp whose lanes are all busy does not ask it
+                few = *(volatile unsigned long long *)A.head >= (unsigned long long)nq &&
+                      nq - (long long)*(volatile unsigned long long *)&A.ws->demoted <= A.handover;
             }
-            give = exhausted && __shfl_sync(FULL, left, 0) <= A.handover;
+            give = __shfl_sync(FULL, (int)few, 0) != 0;
+            exhausted |= give;
         }
         while (!exhausted) {
             const unsigned idle = __ballot_sync(FULL, !has);

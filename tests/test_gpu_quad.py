@@ -129,3 +129,31 @@ def test_budgets_do_not_change_results(side):
     want = records([im], opt, (0,))
     for budgets in ((40, 600, 0), (512, 512, 0), (1024, 1025, 0), (1,) * 5 + (0,)):
         assert np.array_equal(records([im], opt, budgets), want, equal_nan=True), budgets
+
+
+def test_warps_whose_lanes_are_all_busy_hand_over_too():
+    """A warp full of long rays has no idle lane to ask the queue for more; it
+    must still learn that the queue is empty.  Equal rays, whole warps of them,
+    in a buffer of empty slots: all of them are handed over."""
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    n, full = 300 * sms, 32 * (20 * sms // 32)
+    opt = gray.Options(precision=gray.FP64, max_steps=20000)
+    one = torch.tensor([[3.0, 2.0, 0.9, 1.2, 1000.0]], dtype=torch.float64, device="cuda")
+    tr = gray.Tracer(opt, 1)
+    tr.setup_rays(one)
+    tr.trace()
+    want = tr.records()
+    tr.close()
+    tr = gray.Tracer(opt, n)
+    gray.gray_clear(tr.ctx, tr.state, n, 0, n)
+    tr.setup_rays(one.repeat(full, 1), first_ray=0)
+    plane = lambda size: (size * n + 255) // 256 * 256
+    first = 4 * plane(32) + 2 * plane(16)
+    listed = tr.state[first:first + 4 * n].view(torch.int32)
+    listed.fill_(-1)
+    _, n_active, _ = tr.trace()
+    rec = tr.records(first_ray=0, n=full)
+    rays = listed.cpu().numpy()
+    tr.close()
+    assert n_active == 0 and np.all(rec == want)
+    assert np.array_equal(np.sort(rays[rays >= 0]), np.arange(full))
