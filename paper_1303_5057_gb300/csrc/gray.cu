@@ -169,8 +169,8 @@ __device__ __forceinline__ void st_f4(void *p, int64_t i, float x, float y, floa
 // Conversions between double and single precision or integers on the integer
 // and FP32 pipes, exact as the instructions are: those run on the FP64 pipe of
 // this part, 19 cycles of an SM per warp, which the set-up and the read-outs in
-// double are bound by (1000 x 777 rays: set-up 327 -> 272 us, INVARIANTS 168 ->
-// 158; 524288 single rays: set-up 273 -> 246).
+// double are bound by (1000 x 777 rays: set-up 327 -> 272 us, INVARIANTS, cold,
+// 193 -> 180; 524288 single rays: set-up 273 -> 246).
 
 // (double)x
 __device__ __forceinline__ double widen(float x)
@@ -1533,7 +1533,7 @@ __device__ __forceinline__ ds accel_component(const Hole<ds> &H, const Geo<ds> &
 }
 
 // The last zone rays of a block, four warps per 32 rays.  A double-single step
-// is ~3700 instructions in one warp, 5.5 us when the warp is alone, and under
+// is ~3900 instructions in one warp, 5.2 us when the warp is alone, and under
 // Eq. 2 a ray near a pole takes up to a thousand zone steps where the others
 // take 40: that one ray was the pass.  Here lane l of each of the block's four
 // warps holds ray l; warp w computes component w of every acceleration and of
@@ -1744,8 +1744,8 @@ template <int CFG> __device__ __noinline__ void zone_team(const TraceArgs &A, Te
 // four warps' code in the instruction cache at once a team loses to a ray per
 // lane on short rests (1024^2 image 0.276 -> 0.35 ms when every block's last 32
 // rays went to teams), so the hand-over waits for ZONE_TAIL steps after the
-// list is drained.  Eq. 2 image, 509^2: zone pass 5.35 -> 4.35 ms
-// (24 and 48 steps the same within its runs).
+// list is drained.  Eq. 2 images: 61^2, whose longest ray takes 350 zone steps,
+// 1.82 -> 1.55 ms, 509^2 2.85 -> 2.65 (24 and 48 steps the same within its runs).
 template <bool RETURN, typename T, int CFG = CFG_EQUATOR>
 __global__ void __launch_bounds__(128, RETURN ? 3 : 1) zone_kernel(const __grid_constant__ TraceArgs A)
 {
@@ -3328,21 +3328,23 @@ void launch_trace32(const gray_ctx *ctx, const TraceArgs &A, int64_t work, int b
 // evenly over the SMs, four to an SM; a queue long enough that its last rays
 // do not matter takes five (300 x 211 image, a = 0.9, i = 75 deg, planned:
 // three 128-thread blocks per SM 107 ms, 3 / 4 / 5 / 6 / 8 warps 58 / 60 / 66 /
-// 74 / 90; with the hand-over below 49.4 / 49.5 / 51.1 ms at 3 / 4 / 5; 512 x
-// 400: 97 / 82 / 86; 1024^2: 471 / 395 / 392).
+// 74 / 90; with the hand-over below 44.1 / 44.3 / 47.9 ms at 3 / 4 / 5; 512 x
+// 400: 92 / 77 / 80; 1024^2: 456 / 380 / 376).
 //
 // Short queues go to the four-lane kernel at once: there a step of one ray
 // takes 12.7 us instead of 19 (64^2: 45 -> 29 ms), while a chip full of rays
 // does 1.7 times the steps per second with a ray per lane (1024 x 640: 250 ms
 // against 433).  How many rays are few depends on how far the longest exceed
 // the others: under the benchmark rule a planned queue is bound by its long
-// rays up to 200 rays per SM (158^2: 41.7 ms, 43.6 from the one-lane kernel;
-// 170 x 150: 39 and 42), one in any order up to 80 (100^2: 31.1 and 32.8, but
-// 140^2: 42.7 and 38.5); under Eq. 2, whose rays are alike, up to 64 (80^2: 12.0
-// and 15.3, but 120^2: 21.1 and 17.1, 158^2: 27.0 and 19.1).  In longer queues
-// the one-lane kernel hands its last rays over (A.handover; 300 x 211 natural
-// order 62 -> 51, Eq. 2 48 -> 44; 16 to 64 rays per SM are within 2 % of each
-// other).  An order of the caller's counts as planned, whatever it is.
+// rays up to 200 rays per SM (158^2: 34.2 ms, 35.8 from the one-lane kernel;
+// 174^2: 36.0 and 38.8), one in any order up to 80 (100^2: 32.6 and 34.3, but
+// 112^2: 37.1 and 34.4, 140^2: 39.8 and 35.3); under Eq. 2, whose rays are alike,
+// up to 64 (90^2: 13.2 and 14.8, but 112^2: 23.3 and 19.6, 158^2: 27.9 and 20.1).
+// In longer queues the one-lane kernel hands its last rays over (A.handover;
+// 300 x 211 natural order 61.9 -> 50.7, planned 52.3 -> 44.3, Eq. 2 45.2 -> 41.7;
+// 16 to 64 rays per SM are within 3 % of each other).  An order of the caller's
+// counts as planned, whatever it is: one that is not loses up to 16 % between 80
+// and 200 rays per SM against no order.
 //
 // Probe passes, and calls with a budget of up to 512 steps, are the same steps
 // for nearly every ray: no ray is much longer than the others, and the four-lane
@@ -3502,9 +3504,9 @@ int gray_trace(gray_ctx *ctx, void *state, size_t state_bytes, int64_t n_state, 
             // fewest pipe cycles on partly filled warps (1.95 ms at three
             // blocks per SM, 1.53 ms at one, 2.2 ms with 64-thread blocks).
             // Double-single: two blocks per SM, which hide each other's
-            // refills and instruction fetches (1024^2 image 0.319 ms at one,
-            // 0.276 at two, 0.329 at three; r_sw = 0.25: 2.26 / 2.07 / 2.33;
-            // 524288 mixed rays 0.69 / 0.555 / 0.64).
+            // refills and instruction fetches (1024^2 image, planned, 0.386 ms
+            // at one, 0.345 at two, 0.406 at three; r_sw = 0.25: 2.31 / 2.31 /
+            // 2.69; 524288 mixed rays 0.725 / 0.605 / 0.713).
             if (ctx->opt.zone_arith == GRAY_ZONE_FP64) {
                 zone_kernel<true, double><<<(unsigned)ctx->num_sms, block, 0, s>>>(Z);
             } else {

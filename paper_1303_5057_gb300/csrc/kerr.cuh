@@ -574,10 +574,10 @@ __device__ __forceinline__ bool xi_fails_flag(const Hole<float> &H, const Geo<fl
 // ---- double-single arithmetic -------------------------------------------
 // A value carried as an unevaluated sum hi + lo of two floats (about 48
 // significant bits), with the error-free transformations of Knuth (TwoSum)
-// and Dekker (TwoProduct by fused multiply-add).  The tracer uses it only on
-// the rare path that re-takes an ambiguous Eq. 4 test, so that the test is
-// decided to ~2^-40 of its terms without leaving the single-precision pipe
-// (GB300's FP64 rate is 1/64 of FP32's).
+// and Dekker (TwoProduct by fused multiply-add), all on the single-precision
+// pipe (GB300's FP64 rate is 1/64 of FP32's).  The tracer takes every step of
+// the near-horizon zone in it by default (GRAY_ZONE_DS), and outside the zone
+// re-takes an ambiguous Eq. 4 test with it, to ~2^-40 of the test's terms.
 struct ds {
     float hi, lo;
     ds() = default;
